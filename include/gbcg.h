@@ -117,7 +117,7 @@ typedef struct {
   int64_t n;                  /* rows */
   int64_t nnz_input;          /* entries passed to gbcg_create */
   int64_t nnz_full;           /* entries of the full symmetric operator */
-  int64_t stored_slots;       /* SELL slots of the row-gather layout, padding included */
+  int64_t stored_slots;       /* stored value slots of the layout, padding included */
   int64_t plan_slots;         /* SELL slots of the symmetric transpose plan (0 if none) */
   int64_t long_rows;          /* rows handled warp-per-row */
   int64_t device_bytes;       /* device memory held by the handle */
@@ -127,8 +127,10 @@ typedef struct {
   int64_t ext_slots;          /* symmetric tiles: partial sums leaving the tiles */
   int32_t format;             /* gbcg_format */
   int32_t grid_ctas;          /* CTAs of the persistent CG launch */
-  int32_t layout;             /* 0 row gather, 1 symmetric transpose plan, 2 symmetric tiles */
-  int32_t tiles;              /* symmetric tiles: number of tiles */
+  int32_t layout;             /* family: 0 full storage (row gather, or diagonals where the matrix
+                                 has few), 1 symmetric transpose plan, 2 default symmetric storage
+                                 (tiles, or diagonals) */
+  int32_t tiles;              /* symmetric tiles: number of tiles (0 on diagonals) */
   int32_t index_bytes;        /* bytes per column index in the product's stream: 2 when the
                                  row-gather layout stores 16-bit offsets from the row (every
                                  offset fits; natural-order finite-element matrices up to
@@ -159,9 +161,13 @@ typedef struct {
  *   memory     gbcg_memory: where ptr/idx/val live
  *   stream     used for the uploads
  *
- * The library deep-copies the arrays into its own device layout (a sliced
- * row-gather layout for the product, a single-precision copy of the values,
- * the solve workspace); the caller may free its arrays when the call returns.
+ * The library deep-copies the arrays into its own device layout (values by
+ * diagonal when the matrix has at most 32 diagonals that are at least two
+ * thirds full, as a mesh numbered line by line gives; else a sliced row-gather
+ * layout or symmetric tiles; a single-precision copy of the values, the solve
+ * workspace); the caller may free its arrays when the call returns.  The
+ * environment variables GBCG_DIAGONALS=0 and GBCG_SYM_LAYOUT=tiles|plan keep
+ * the other layouts.
  * Errors: GBCG_ERR_INVALID for malformed input (with the first offending
  * position in gbcg_last_error()), GBCG_ERR_NOMEM, GBCG_ERR_CUDA.
  */

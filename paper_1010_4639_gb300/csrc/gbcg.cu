@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "../../include/gbcg.h"
+#include "dia_solve.cuh"
 #include "kernels.cuh"
 #include "layout.h"
 
@@ -63,6 +64,17 @@ int upload(T** p, const std::vector<T>& h, cudaStream_t s, int64_t& bytes) {
 std::vector<float> to_f32(const std::vector<double>& v) {
   std::vector<float> o(v.size());
   for (size_t i = 0; i < v.size(); ++i) o[i] = (float)v[i];
+  return o;
+}
+
+// Single-precision copy of a diagonal layout's values: only its padding stays
+// -0.0 (an entry may round to zero).
+std::vector<float> dia_to_f32(const std::vector<double>& v) {
+  std::vector<float> o(v.size());
+  for (size_t i = 0; i < v.size(); ++i) {
+    const bool padding = v[i] == 0.0 && std::signbit(v[i]);
+    o[i] = padding ? -0.f : dia_value((float)v[i]);
+  }
   return o;
 }
 
@@ -200,12 +212,18 @@ struct gbcg_matrix_s {
   double* u_stage = nullptr;
   int64_t nslices = 0, nlong = 0, bytes = 0;
   int sym = 0;
-  int mode = kGather;       // kGather (CSR/CSC), kPlan or kTiles (symmetric)
+  int mode = kGather;       // kGather or kDia (CSR/CSC), kPlan, kTiles or kDiaSym (symmetric)
   int64_t l2_bytes = 0;     // the device's L2 size
   // tiled symmetric layouts (device): single- and double-precision products
   DevTiles t32, t64;
   int32_t *u_map_t32 = nullptr;  // value map of the single-precision tiles (u_map_main: double-precision)
   int64_t u_len_t32 = 0;
+  // diagonal layout (kDia, kDiaSym)
+  std::vector<int32_t> dia_off;
+  int64_t dia_ld = 0;
+  double* dia64 = nullptr;
+  float* dia32 = nullptr;
+  bool narrow = false;       // every column offset fits 16 bits
   // layout (device)
   int64_t* sl_ptr = nullptr;
   int32_t* col = nullptr;
@@ -228,6 +246,8 @@ struct gbcg_matrix_s {
   int32_t* cta_slice = nullptr;
   int32_t* cta_long = nullptr;
   // workspace
+  double *p_base = nullptr;  // p within its halo (diagonal layout)
+  float* p32_base = nullptr;
   double *r = nullptr, *p = nullptr, *q = nullptr, *bstage = nullptr, *xstage = nullptr;
   float *r32 = nullptr, *p32 = nullptr, *q32 = nullptr, *d32 = nullptr, *rhs32 = nullptr;
   // single-reduction CG (double precision): s = A p, z = A s, w = A r (two buffers)
@@ -235,8 +255,10 @@ struct gbcg_matrix_s {
   double* part = nullptr;   // max(2 * grid, one-shot blocks)
   double* sums = nullptr;   // small scalars
   int64_t part_len = 0;
-  GridBar* bar = nullptr;
+  ChipSync* sync = nullptr;
+  GridBar* bar = nullptr;   // &sync->bar
   CgState* st = nullptr;
+  int64_t chip_rows = 0;    // diagonal layout: greatest number of rows of a CTA
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // brackets of the persistent launches
   // pinned host mirrors
   CgState* st_h = nullptr;
@@ -248,6 +270,20 @@ struct gbcg_matrix_s {
   template <typename V>
   SymDev<V> tiles() const {
     return sizeof(V) == 4 ? t32.dev<V>() : t64.dev<V>();
+  }
+  template <typename V>
+  DiaDev<V> dia() const {
+    DiaDev<V> d;
+    if (dia_off.empty()) return d;
+    d.n = n;
+    d.ld = dia_ld;
+    if constexpr (sizeof(V) == 4) d.val = dia32;
+    else d.val = dia64;
+    d.K = (int32_t)dia_off.size();
+    std::copy(dia_off.begin(), dia_off.end(), d.off);
+    d.hi = dia_off.back();
+    d.lo = mode == kDiaSym ? -d.hi : dia_off.front();
+    return d;
   }
   int spmv_blocks() const { return (int)std::max<int64_t>(1, (nslices + nlong + 7) / 8); }
 };
@@ -301,9 +337,9 @@ void free_matrix(gbcg_matrix_s* M) {
   if (!M) return;
   void* dev[] = {M->sl_ptr, M->col, M->col16, M->val64, M->val32, M->long_mask, M->long_row, M->long_ptr, M->long_col,
                  M->long_val64, M->long_val32, M->diag64, M->diag32, M->pl_ptr, M->pl_i, M->pl_k,
-                 M->cta_slice, M->cta_long, M->r, M->p, M->q, M->bstage, M->xstage, M->r32, M->p32, M->q32,
-                 M->d32, M->rhs32, M->part, M->sums, M->bar, M->st, M->u_map_main, M->u_map_long, M->u_map_diag,
-                 M->u_map_t32, M->u_stage, M->s64, M->z64, M->w64a, M->w64b};
+                 M->cta_slice, M->cta_long, M->r, M->p_base, M->q, M->bstage, M->xstage, M->r32, M->p32_base, M->q32,
+                 M->d32, M->rhs32, M->part, M->sums, M->sync, M->st, M->u_map_main, M->u_map_long, M->u_map_diag,
+                 M->u_map_t32, M->u_stage, M->dia64, M->dia32, M->s64, M->z64, M->w64a, M->w64b};
   M->t32.release();
   M->t64.release();
   for (void* d : dev)
@@ -315,9 +351,6 @@ void free_matrix(gbcg_matrix_s* M) {
   if (M->ev1) cudaEventDestroy(M->ev1);
   delete M;
 }
-
-// Threads per CTA: the tiled symmetric kernels add a producer warp.
-constexpr int block_of(int fmt) { return fmt == kTiles ? kTileThreads : kCgThreads; }
 
 template <typename V, int FMT, bool OUTER>
 int occupancy_of(int& per_sm) {
@@ -332,7 +365,8 @@ int occupancy_of(int& per_sm) {
 // pipelines' carvings, used in turn.
 template <int FMT>
 constexpr size_t ru_smem() {
-  return FMT == kTiles ? std::max(sym_smem_bytes<float>(), sym_smem_bytes<double>())
+  return FMT == kTiles   ? std::max(sym_smem_bytes<float>(), sym_smem_bytes<double>())
+         : is_dia(FMT) ? stream_smem_bytes<4>()
                        : (size_t)kWarps * ru_warp_stage_bytes();
 }
 
@@ -345,20 +379,21 @@ int ru_occupancy_of(int& per_sm) {
 
 template <int FMT>
 int pcg_occupancy_of(int& per_sm) {
-  if constexpr (FMT == kTiles) {
+  if constexpr (FMT == kTiles || FMT == kDiaSym) {  // no single-reduction form on the default symmetric layouts
     per_sm = 1 << 20;
     return 0;
   } else {
     const size_t sm = product_smem<double, FMT>();
     CUDA_TRY(cudaFuncSetAttribute(k_pcg<double, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg<double, FMT>, kCgThreads, sm));
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg<double, FMT>, block_of(FMT), sm));
     return 0;
   }
 }
 
 template <typename V, int FMT>
 int prepare_rows() {
-  CUDA_TRY(cudaFuncSetAttribute(k_rows<V, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if constexpr (is_dia(FMT)) return 0;
+  else CUDA_TRY(cudaFuncSetAttribute(k_rows<V, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)product_smem<V, FMT>()));
   return 0;
 }
@@ -379,8 +414,13 @@ int solver_occupancy(int& per_sm) {
 }
 
 int mode_occupancy(int mode, int& per_sm) {
-  return mode == kTiles ? solver_occupancy<kTiles>(per_sm)
-                        : mode == kPlan ? solver_occupancy<kPlan>(per_sm) : solver_occupancy<kGather>(per_sm);
+  switch (mode) {
+    case kTiles: return solver_occupancy<kTiles>(per_sm);
+    case kPlan: return solver_occupancy<kPlan>(per_sm);
+    case kDia: return solver_occupancy<kDia>(per_sm);
+    case kDiaSym: return solver_occupancy<kDiaSym>(per_sm);
+    default: return solver_occupancy<kGather>(per_sm);
+  }
 }
 
 // The kernels read and write vectors with 16-byte loads and bulk copies.
@@ -407,6 +447,8 @@ cudaError_t launch_cg_fmt(const gbcg_matrix_s* M, const CgArgs<V>& a, cudaStream
   switch (M->mode) {
     case kTiles: return launch_cg<V, kTiles, OUTER>(a, M->grid, s);
     case kPlan: return launch_cg<V, kPlan, OUTER>(a, M->grid, s);
+    case kDia: return launch_cg<V, kDia, OUTER>(a, M->grid, s);
+    case kDiaSym: return launch_cg<V, kDiaSym, OUTER>(a, M->grid, s);
     default: return launch_cg<V, kGather, OUTER>(a, M->grid, s);
   }
 }
@@ -414,12 +456,12 @@ cudaError_t launch_cg_fmt(const gbcg_matrix_s* M, const CgArgs<V>& a, cudaStream
 template <int FMT>
 cudaError_t launch_pcg(const PcgArgs<double>& args, int grid, cudaStream_t s) {
   void* kargs[] = {(void*)&args};
-  return cudaLaunchCooperativeKernel((const void*)k_pcg<double, FMT>, dim3(grid), dim3(kCgThreads), kargs,
+  return cudaLaunchCooperativeKernel((const void*)k_pcg<double, FMT>, dim3(grid), dim3(block_of(FMT)), kargs,
                                      product_smem<double, FMT>(), s);
 }
 
-// The single-reduction CG on the handle's layout (row-gather layouts only;
-// the caller has checked the mode).
+// The single-reduction CG on the handle's layout (not the default symmetric
+// ones; the caller has checked the mode).
 cudaError_t launch_pcg_fmt(const gbcg_matrix_s* M, const CgArgs<double>& c, cudaStream_t s) {
   PcgArgs<double> a;
   a.c = c;
@@ -427,7 +469,9 @@ cudaError_t launch_pcg_fmt(const gbcg_matrix_s* M, const CgArgs<double>& c, cuda
   a.z = M->z64;
   a.w0 = M->w64a;
   a.w1 = M->w64b;
-  return M->mode == kPlan ? launch_pcg<kPlan>(a, M->grid, s) : launch_pcg<kGather>(a, M->grid, s);
+  return M->mode == kPlan  ? launch_pcg<kPlan>(a, M->grid, s)
+         : M->mode == kDia ? launch_pcg<kDia>(a, M->grid, s)
+                           : launch_pcg<kGather>(a, M->grid, s);
 }
 
 template <int FMT>
@@ -437,13 +481,65 @@ cudaError_t launch_ru(const RuArgs& args, int grid, cudaStream_t s) {
                                      ru_smem<FMT>(), s);
 }
 
+// Dynamic shared memory a CTA of the on-chip solvers may take: the opt-in
+// limit less their static variables.
+constexpr size_t kChipSmem = 225 * 1024;
+
+// Whether a CTA's rows of the four vectors fit on the chip (dia_solve.cuh).
+template <typename V>
+bool on_chip(const gbcg_matrix_s* M) {
+  return is_dia(M->mode) && M->grid <= kChipCtas && chip_smem<V>(M->chip_rows, kChipThreads) <= kChipSmem;
+}
+
+template <typename V, bool SYM, int KIND, int R>
+cudaError_t launch_chip(const gbcg_matrix_s* M, ChipArgs<V> a, cudaStream_t s) {
+  a.D = M->dia<V>();
+  a.D64 = M->dia<double>();
+  a.sync = M->sync;
+  a.st = M->st;
+  a.nslices = M->nslices;
+  a.rows = (int32_t)M->chip_rows;
+  const int threads = (int)std::min<int64_t>(chip_threads(R), M->chip_rows);
+  const size_t smem = chip_smem<V>(M->chip_rows, threads);
+  const void* kernel = (const void*)k_dia_chip<V, SYM, KIND, R>;
+  cudaError_t e = cudaMemsetAsync(M->sync, 0, sizeof(ChipSync), s);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChipSmem);
+  if (e != cudaSuccess) return e;
+  void* kargs[] = {(void*)&a};
+  return cudaLaunchCooperativeKernel(kernel, dim3(M->grid), dim3(threads), kargs, smem, s);
+}
+template <typename V, int KIND>
+cudaError_t launch_chip_fmt(const gbcg_matrix_s* M, const ChipArgs<V>& a, cudaStream_t s) {
+  // two rows per thread and product step once 512 threads would take more than
+  // four rounds (1024 threads of 64 registers: 36.1 against 38.1 us per FP64
+  // iteration, 17.7 against 19.3 single precision, at 5 500 rows per CTA; one
+  // row per step and 128 registers for short ranges, where the round trip
+  // counts: 8.5 against 10.5 us at 170 rows)
+  constexpr int R = 2;
+  if (M->chip_rows > 2048)
+    return M->mode == kDiaSym ? launch_chip<V, true, KIND, R>(M, a, s) : launch_chip<V, false, KIND, R>(M, a, s);
+  return M->mode == kDiaSym ? launch_chip<V, true, KIND, 1>(M, a, s) : launch_chip<V, false, KIND, 1>(M, a, s);
+}
+
 // Product y = A x (MODE 0), or r = b - A x into y with per-CTA partial sums
 // of r'r in part (MODE 1, double precision), on the persistent partition.
 template <typename V, int FMT, int MODE>
 cudaError_t launch_product(const gbcg_matrix_s* M, const V* x, const V* b, V* y, cudaStream_t s) {
-  k_rows<V, FMT><<<M->grid, block_of(FMT), product_smem<V, FMT>(), s>>>(
+  if constexpr (is_dia(FMT)) {
+    // four rows per thread in single precision once that leaves two blocks per
+    // SM (128^3: 16 us against 25 with one row; 10 us either way at 64^3); one
+    // in double precision, where more rows per thread only crowd the FP64
+    // pipe's queue (128^3: 60 us against 120 with two)
+    constexpr int R = dia_r<V>();
+    auto blocks = [&](int rows) { return (unsigned)((M->n + rows * kDiaBlock - 1) / (rows * kDiaBlock)); };
+    if (M->n > 300000)
+      k_dia_rows<V, FMT == kDiaSym, R><<<blocks(R), kDiaBlock, 0, s>>>(M->dia<V>(), x, y);
+    else
+      k_dia_rows<V, FMT == kDiaSym, 1><<<blocks(1), kDiaBlock, 0, s>>>(M->dia<V>(), x, y);
+  } else
+    k_rows<V, FMT><<<M->grid, block_of(FMT), product_smem<V, FMT>(), s>>>(
       M->op<V>(), M->tiles<V>(), M->cta_slice, M->cta_long, x, y, &M->bar->status, 1000000000LL);
-  if (FMT == kTiles || MODE == 1)
+  if constexpr (FMT == kTiles || MODE == 1)
     k_finish<V, FMT, MODE><<<M->grid, kCgThreads, 0, s>>>(M->tiles<V>(), M->cta_slice, M->n, b, y, M->part);
   return cudaGetLastError();
 }
@@ -453,6 +549,8 @@ cudaError_t launch_product_fmt(const gbcg_matrix_s* M, const V* x, const V* b, V
   switch (M->mode) {
     case kTiles: return launch_product<V, kTiles, MODE>(M, x, b, y, s);
     case kPlan: return launch_product<V, kPlan, MODE>(M, x, b, y, s);
+    case kDia: return launch_product<V, kDia, MODE>(M, x, b, y, s);
+    case kDiaSym: return launch_product<V, kDiaSym, MODE>(M, x, b, y, s);
     default: return launch_product<V, kGather, MODE>(M, x, b, y, s);
   }
 }
@@ -502,6 +600,7 @@ CgArgs<V> make_args(const gbcg_matrix_s* M, V* x, V* r, V* p, V* q, const V* b, 
   CgArgs<V> a;
   a.A = M->op<V>();
   a.T = M->tiles<V>();
+  a.D = M->dia<V>();
   a.x = x;
   a.r = r;
   a.p = p;
@@ -543,7 +642,21 @@ cudaError_t enqueue_fp64(gbcg_matrix_s* M, const double* b, double* x, double to
   if (e != cudaSuccess) return e;
   CgArgs<double> a = make_args<double>(M, x, M->r, M->p, M->q, b, tol, maxit, max_restarts, timeout_ns_of(o));
   if (timed && (e = cudaEventRecord(M->ev0, s)) != cudaSuccess) return e;
-  e = (o && o->variant == GBCG_PIPELINED) ? launch_pcg_fmt(M, a, s) : launch_cg_fmt<double, true>(M, a, s);
+  if (o && o->variant == GBCG_PIPELINED) {
+    e = launch_pcg_fmt(M, a, s);
+  } else if (on_chip<double>(M)) {
+    ChipArgs<double> ca = {};
+    ca.x = x;
+    ca.b = b;
+    ca.p = M->p;
+    ca.tol = tol;
+    ca.maxit = maxit;
+    ca.max_restarts = max_restarts;
+    ca.timeout_ns = a.timeout_ns;
+    e = launch_chip_fmt<double, kSolveFull>(M, ca, s);
+  } else {
+    e = launch_cg_fmt<double, true>(M, a, s);
+  }
   if (e != cudaSuccess) return e;
   return timed ? cudaEventRecord(M->ev1, s) : cudaSuccess;
 }
@@ -580,14 +693,31 @@ cudaError_t enqueue_ru(gbcg_matrix_s* M, const double* b, double* x, double tol,
   a.c = make_args<float>(M, M->d32, M->r32, M->p32, M->q32, nullptr, tol, maxit, 0, timeout_ns_of(o));
   a.A64 = M->op<double>();
   a.T64 = M->tiles<double>();
+  a.D64 = M->dia<double>();
   a.x64 = x;
   a.b64 = b;
   a.q64 = M->q;
   a.delta = (o && o->inner_tol > 0.0 && o->inner_tol < 1.0) ? o->inner_tol : 0.1;
   if (timed && (e = cudaEventRecord(M->ev0, s)) != cudaSuccess) return e;
-  e = M->mode == kTiles  ? launch_ru<kTiles>(a, M->grid, s)
-      : M->mode == kPlan ? launch_ru<kPlan>(a, M->grid, s)
-                         : launch_ru<kGather>(a, M->grid, s);
+  if (on_chip<float>(M)) {
+    ChipArgs<float> ca = {};
+    ca.p = M->p32;
+    ca.x64 = x;
+    ca.b64 = b;
+    ca.xh = M->p;
+    ca.tol = tol;
+    ca.delta = a.delta;
+    ca.maxit = maxit;
+    ca.timeout_ns = a.c.timeout_ns;
+    e = launch_chip_fmt<float, kSolveRu>(M, ca, s);
+  } else
+  switch (M->mode) {
+    case kTiles: e = launch_ru<kTiles>(a, M->grid, s); break;
+    case kPlan: e = launch_ru<kPlan>(a, M->grid, s); break;
+    case kDia: e = launch_ru<kDia>(a, M->grid, s); break;
+    case kDiaSym: e = launch_ru<kDiaSym>(a, M->grid, s); break;
+    default: e = launch_ru<kGather>(a, M->grid, s); break;
+  }
   if (e != cudaSuccess) return e;
   return timed ? cudaEventRecord(M->ev1, s) : cudaSuccess;
 }
@@ -664,7 +794,18 @@ int solve_ir(gbcg_matrix_s* M, const double* b, double* x, double tol, int maxit
       CUDA_TRY(cudaMemsetAsync(M->bar, 0, sizeof(GridBar), s));
       CgArgs<float> a = make_args<float>(M, M->d32, M->r32, M->p32, M->q32, M->rhs32, inner_tol, maxit - used, 0, tns);
       CUDA_TRY(cudaEventRecord(M->ev0, s));
-      CUDA_TRY(launch_cg_fmt<float, false>(M, a, s));
+      if (on_chip<float>(M)) {
+        ChipArgs<float> ca = {};
+        ca.x = M->d32;
+        ca.b = M->rhs32;
+            ca.p = M->p32;
+        ca.tol = inner_tol;
+        ca.maxit = maxit - used;
+        ca.timeout_ns = tns;
+        CUDA_TRY(launch_chip_fmt<float, kSolveInner>(M, ca, s));
+      } else {
+        CUDA_TRY(launch_cg_fmt<float, false>(M, a, s));
+      }
       CUDA_TRY(cudaEventRecord(M->ev1, s));
       if (int rc = read_state(M, s)) return rc;
       float kms = 0.f;
@@ -737,9 +878,17 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
     val = hval.data();
   }
   LayoutHost L;
+  DiaHost Dh;
   std::string err;
-  int rc = build_layout(format, n, nnz, ptr, idx, val, index_base, L, err);
+  int rc = validate_input(format, n, nnz, ptr, idx, val, index_base, err);
   if (rc) return fail(rc, err);
+  // a matrix of few diagonals takes the diagonal layout (layout.h has the
+  // rule); a layout asked for by name, or GBCG_DIAGONALS=0, keeps the others
+  const char* sym_mode = getenv("GBCG_SYM_LAYOUT");
+  const bool sym_named = format == GBCG_SYM_CSR_UPPER && sym_mode && *sym_mode;
+  const bool diagonals = !sym_named && env_int("GBCG_DIAGONALS", 1) != 0 &&
+                         build_diagonals(format, n, nnz, ptr, idx, val, index_base, Dh);
+  if (!diagonals && (rc = build_layout(format, n, nnz, ptr, idx, val, index_base, L, err)) != 0) return fail(rc, err);
   // debug mode: full CSR/CSC inputs must be symmetric (CG's premise)
   if (format != GBCG_SYM_CSR_UPPER && env_int("GBCG_CHECK_SYMMETRY", 0) != 0 &&
       (rc = check_symmetry(n, nnz, ptr, idx, val, index_base, err)) != 0)
@@ -749,11 +898,11 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
   M->format = format;
   M->n = n;
   M->nnz_input = nnz;
-  M->nnz_full = L.nnz_full;
+  M->nnz_full = diagonals ? Dh.nnz_full : L.nnz_full;
   M->sym = format == GBCG_SYM_CSR_UPPER;
-  M->nslices = L.A.nslices;
+  M->nslices = (n + 31) / 32;
   M->nlong = (int64_t)L.A.long_row.size();
-  M->slots = L.A.sl_ptr.empty() ? 0 : L.A.sl_ptr.back();
+  M->slots = diagonals ? (int64_t)Dh.val.size() : L.A.sl_ptr.empty() ? 0 : L.A.sl_ptr.back();
   M->plan_slots = L.plan.pl_ptr.empty() ? 0 : L.plan.pl_ptr.back();
   M->index_base = index_base;
   M->h_ptr.assign(ptr, ptr + n + 1);
@@ -777,8 +926,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
     return bail(fail(GBCG_ERR_CUDA, "cannot query the device"));
   M->l2_bytes = l2;
-  const char* sym_mode = getenv("GBCG_SYM_LAYOUT");
-  M->mode = !M->sym ? kGather : (sym_mode && !strcmp(sym_mode, "plan")) ? kPlan : kTiles;
+  M->mode = diagonals ? (M->sym ? kDiaSym : kDia) : !M->sym ? kGather : (sym_mode && !strcmp(sym_mode, "plan")) ? kPlan : kTiles;
   auto choose_grid = [&]() -> int {
     if (int rc = mode_occupancy(M->mode, per_sm)) return rc;
     if (per_sm < 1) return fail(GBCG_ERR_CUDA, "the persistent solver kernel cannot be resident");
@@ -812,11 +960,21 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
     M->slots = M->t64.slots;
     M->plan_slots = 0;
     TRY(upload(&M->long_mask, std::vector<uint32_t>(std::max<int64_t>(M->nslices, 1), 0u), s, B));
+  } else if (diagonals) {
+    M->dia_off = Dh.off;
+    M->dia_ld = Dh.ld;
+    M->narrow = !M->sym && Dh.off.front() >= -32768 && Dh.off.back() <= 32767 && env_int("GBCG_WIDE_INDEX", 0) == 0;
+    TRY(upload(&M->dia64, Dh.val, s, B));
+    TRY(upload(&M->dia32, dia_to_f32(Dh.val), s, B));
+    // every row costs the same: equal ranges of whole slices
+    cs.resize(M->grid + 1);
+    for (int c = 0; c <= M->grid; ++c) cs[c] = (int32_t)(chip_row(M->nslices, c, M->grid) / 32);
+    for (int c = 0; c < M->grid; ++c) M->chip_rows = std::max<int64_t>(M->chip_rows, 32 * (int64_t)(cs[c + 1] - cs[c]));
   } else {
     TRY(upload(&M->sl_ptr, L.A.sl_ptr, s, B));
     TRY(upload(&M->col, L.A.col, s, B));
-    if (!L.A.col16.empty() && M->mode == kGather && env_int("GBCG_WIDE_INDEX", 0) == 0)
-      TRY(upload(&M->col16, L.A.col16, s, B));
+    M->narrow = !L.A.col16.empty() && M->mode == kGather && env_int("GBCG_WIDE_INDEX", 0) == 0;
+    if (M->narrow) TRY(upload(&M->col16, L.A.col16, s, B));
     TRY(upload(&M->val64, L.A.val, s, B));
     TRY(upload(&M->val32, to_f32(L.A.val), s, B));
     TRY(upload(&M->long_mask, L.A.long_mask, s, B));
@@ -837,7 +995,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
     }
     cl[M->grid] = (int32_t)M->nlong;
   }
-  if (M->sym) {
+  if (M->sym && !diagonals) {
     TRY(upload(&M->diag64, L.diag, s, B));
     TRY(upload(&M->diag32, to_f32(L.diag), s, B));
   }
@@ -846,16 +1004,23 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
   // workspace
   const size_t nn = (size_t)std::max<int64_t>(n, 1);
   TRY(dalloc(&M->r, nn, B));
-  TRY(dalloc(&M->p, nn, B));
+  // the diagonal layout's product reads p beyond its ends (padding values there): zeros that stay zeros
+  const size_t halo = !diagonals ? 0 : (std::max<int64_t>(-M->dia<double>().lo, M->dia<double>().hi) + kDiaHalo + 63) & ~int64_t(63);
+  TRY(dalloc(&M->p_base, nn + 2 * halo, B));
+  TRY(dalloc(&M->p32_base, nn + 2 * halo, B));
+  if (cudaMemsetAsync(M->p_base, 0, sizeof(double) * (nn + 2 * halo), s) != cudaSuccess ||
+      cudaMemsetAsync(M->p32_base, 0, sizeof(float) * (nn + 2 * halo), s) != cudaSuccess)
+    return bail(fail(GBCG_ERR_CUDA, "cudaMemsetAsync failed"));
+  M->p = M->p_base + halo;
+  M->p32 = M->p32_base + halo;
   TRY(dalloc(&M->q, nn, B));
   TRY(dalloc(&M->bstage, nn, B));
   TRY(dalloc(&M->xstage, nn, B));
   TRY(dalloc(&M->r32, nn, B));
-  TRY(dalloc(&M->p32, nn, B));
   TRY(dalloc(&M->q32, nn, B));
   TRY(dalloc(&M->d32, nn, B));
   TRY(dalloc(&M->rhs32, nn, B));
-  if (M->mode != kTiles) {  // the single-reduction CG's vectors
+  if (M->mode != kTiles && M->mode != kDiaSym) {  // the single-reduction CG's vectors
     TRY(dalloc(&M->s64, nn, B));
     TRY(dalloc(&M->z64, nn, B));
     TRY(dalloc(&M->w64a, nn, B));
@@ -864,7 +1029,8 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
   M->part_len = std::max<int64_t>({6 * (int64_t)M->grid, (int64_t)M->spmv_blocks(), 4096});
   TRY(dalloc(&M->part, (size_t)M->part_len, B));
   TRY(dalloc(&M->sums, 8, B));
-  TRY(dalloc(&M->bar, 1, B));
+  TRY(dalloc(&M->sync, 1, B));
+  M->bar = &M->sync->bar;
   TRY(dalloc(&M->st, 1, B));
   if (cudaMallocHost((void**)&M->st_h, sizeof(CgState)) != cudaSuccess ||
       cudaMallocHost((void**)&M->bar_h, sizeof(GridBar)) != cudaSuccess ||
@@ -907,7 +1073,7 @@ int check_solve_opts(const gbcg_matrix_s* A, const gbcg_opts* opts) {
     return fail(GBCG_ERR_INVALID,
                 "the single-reduction variant is double precision only: in single precision its recurrences "
                 "drift past any useful inner tolerance");
-  if (opts && opts->variant == GBCG_PIPELINED && A->mode == kTiles)
+  if (opts && opts->variant == GBCG_PIPELINED && (A->mode == kTiles || A->mode == kDiaSym))
     return fail(GBCG_ERR_INVALID,
                 "the single-reduction variant runs on row-gather layouts (CSR, CSC, or symmetric storage with "
                 "GBCG_SYM_LAYOUT=plan); the tiled symmetric product needs a barrier of its own");
@@ -1000,13 +1166,13 @@ int gbcg_stats(gbcg_matrix_t A, gbcg_matrix_stats* out) {
   const int64_t n = A->n, m = A->nnz_input;
   // the product's matrix stream: value + column index per entry (2-byte
   // offsets in the row-gather layout when they fit), row pointers, x, y
-  const int64_t ib = A->col16 ? 2 : 4;
+  const int64_t ib = A->narrow ? 2 : 4;
   out->spmv_bytes_fp64 = (8 + ib) * m + 4 * (n + 1) + 16 * n;
   out->spmv_bytes_fp32 = (4 + ib) * m + 4 * (n + 1) + 8 * n;
   out->index_bytes = (int32_t)ib;
   out->format = A->format;
   out->grid_ctas = A->grid;
-  out->layout = A->mode;
+  out->layout = A->mode == kDia ? kGather : A->mode == kDiaSym ? kTiles : A->mode;
   out->tiles = (int32_t)A->t64.ntiles;  // the double-precision layout's (the single-precision one has about half)
   out->ext_slots = A->t64.next;
   return GBCG_OK;
@@ -1025,10 +1191,17 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
     // device value slot then names the input entry it holds (0: padding)
     std::vector<double> iv(nnz);
     for (int64_t k = 0; k < nnz; ++k) iv[k] = (double)(k + 1);
+    const bool diagonals = A->mode == kDia || A->mode == kDiaSym;
     LayoutHost L;
+    DiaHost Dh;
     std::string err;
-    if (int rc = build_layout(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, L, err))
+    if (diagonals) {
+      if (!build_diagonals(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, Dh))
+        return fail(GBCG_ERR_INVALID, "rebuilding the value map: diagonals differ from the handle's");
+    } else if (int rc = build_layout(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base,
+                                     L, err)) {
       return fail(rc, "rebuilding the value map: " + err);
+    }
     SymTilesHost T32, T64;
     if (A->mode == kTiles &&
         (!build_sym_tiles(L, A->grid, TileCaps<float>::kSlot, TileCaps<float>::kEnt, kTileSlices32, T32) ||
@@ -1047,6 +1220,9 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
       A->u_len_main = (int64_t)T64.val.size();
       if (int rc = upload(&A->u_map_t32, to_map(T32.val), s, B)) return rc;
       A->u_len_t32 = (int64_t)T32.val.size();
+    } else if (diagonals) {
+      if (int rc = upload(&A->u_map_main, to_map(Dh.val), s, B)) return rc;
+      A->u_len_main = (int64_t)Dh.val.size();
     } else {
       if (int rc = upload(&A->u_map_main, to_map(L.A.val), s, B)) return rc;
       A->u_len_main = (int64_t)L.A.val.size();
@@ -1055,7 +1231,7 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
         A->u_len_long = (int64_t)L.A.long_val.size();
       }
     }
-    if (A->sym) {
+    if (A->sym && !diagonals) {
       if (int rc = upload(&A->u_map_diag, to_map(L.diag), s, B)) return rc;
       A->u_len_diag = (int64_t)L.diag.size();
     }
@@ -1069,18 +1245,20 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
   auto run = [&](const int32_t* map, int64_t len, double* d64, float* d32) -> int {
     if (!map || len == 0) return 0;
     const int blocks = (int)std::min<int64_t>(4096, (len + 255) / 256);
-    k_place_values<<<blocks, 256, 0, s>>>(map, len, src, d64, d32);
+    k_place_values<<<blocks, 256, 0, s>>>(map, len, src, d64, d32, A->mode == kDia || A->mode == kDiaSym);
     CUDA_TRY(cudaGetLastError());
     return 0;
   };
   if (A->mode == kTiles) {
     if (int rc = run(A->u_map_main, A->u_len_main, (double*)A->t64.val, nullptr)) return rc;
     if (int rc = run(A->u_map_t32, A->u_len_t32, nullptr, (float*)A->t32.val)) return rc;
+  } else if (A->mode == kDia || A->mode == kDiaSym) {
+    if (int rc = run(A->u_map_main, A->u_len_main, A->dia64, A->dia32)) return rc;
   } else {
     if (int rc = run(A->u_map_main, A->u_len_main, A->val64, A->val32)) return rc;
     if (int rc = run(A->u_map_long, A->u_len_long, A->long_val64, A->long_val32)) return rc;
   }
-  if (A->sym)
+  if (A->sym && A->u_map_diag)
     if (int rc = run(A->u_map_diag, A->u_len_diag, A->diag64, A->diag32)) return rc;
   return GBCG_OK;
 }

@@ -32,6 +32,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "diagonals.cuh"
 #include "layout.h"  // TileDesc: the packed per-tile descriptor of the tiled symmetric layout
 
 #include <type_traits>
@@ -52,7 +53,10 @@ constexpr uint16_t kPlanPad = 0xFFFF;
 constexpr int kMaxStages = 3 + 2;  // mbarriers per warp: a single- (3) and a double-precision (2) pipeline
 
 // Layout modes of the product.
-enum { kGather = 0, kPlan = 1, kTiles = 2 };
+enum { kGather = 0, kPlan = 1, kTiles = 2, kDia = 3, kDiaSym = 4 };
+__host__ __device__ constexpr bool is_dia(int fmt) { return fmt == kDia || fmt == kDiaSym; }
+// Threads per CTA of the persistent kernels in a layout mode.
+__host__ __device__ constexpr int block_of(int fmt) { return is_dia(fmt) ? kDiaThreads : kCgThreads; }
 
 enum DevStatus { kOk = 0, kNotSpd = 2, kMaxit = 3, kNonfinite = 4, kTimeout = 5 };
 
@@ -128,6 +132,7 @@ template <typename V>
 struct CgArgs {
   OpDev<V> A;
   SymDev<V> T;
+  DiaDev<V> D;
   V* x;
   V* r;
   V* p;
@@ -1043,11 +1048,20 @@ __device__ __forceinline__ bool grid_barrier(GridBar* gb, unsigned long long& ta
   return *sflag != 0;
 }
 
+// Streamed vector passes (stream_rows below): chunk size and depth.
+constexpr int kVecChunkBytes = 8192;  // per array and chunk
+constexpr int kVecBufs = 4;           // chunks in flight
+template <int NA>
+__host__ __device__ constexpr size_t stream_smem_bytes() { return (size_t)kVecBufs * NA * kVecChunkBytes; }
+
 // -------------------------------------------------- one-shot kernels ---
 // Shared-memory carving of the product kernels for layout mode FMT.
 template <typename V, int FMT>
 constexpr size_t product_smem() {
-  return FMT == kGather ? pipe_smem_bytes<V>() : FMT == kTiles ? sym_smem_bytes<V>() : 0;
+  return FMT == kGather                     ? pipe_smem_bytes<V>()
+         : FMT == kTiles                    ? sym_smem_bytes<V>()
+         : is_dia(FMT) && sizeof(V) == 4 ? stream_smem_bytes<4>()
+                                            : 0;
 }
 
 // Computes A x into y for the CTA's rows: complete for kGather / kPlan; for
@@ -1069,7 +1083,7 @@ __device__ __forceinline__ void product_rows(const OpDev<V>& A, const SymDev<V>&
 
 // y = A x on the persistent grid's partition (first pass for kTiles).
 template <typename V, int FMT>
-__global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1)
+__global__ void __launch_bounds__(block_of(FMT), 1)
     k_rows(OpDev<V> A, SymDev<V> T, const int32_t* __restrict__ cta_slice, const int32_t* __restrict__ cta_long,
            const V* __restrict__ x, V* __restrict__ y, int* err, long long limit_ns) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1143,14 +1157,20 @@ __global__ void k_scale_to_f32(const double* __restrict__ r, double scale, int64
 
 // Value update of a handle: slot i of a device value array takes input
 // value map[i] (0 where map[i] < 0: padding), in double precision into d64
-// and in single precision into d32 (either may be null).
+// and in single precision into d32 (either may be null).  dia: the diagonal
+// layout's stored forms (padding -0.0, zeros +0.0).
 __global__ void k_place_values(const int32_t* __restrict__ map, int64_t len, const double* __restrict__ src,
-                               double* __restrict__ d64, float* __restrict__ d32) {
+                               double* __restrict__ d64, float* __restrict__ d32, bool dia) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t k = map[i];
     const double v = k >= 0 ? src[k] : 0.0;
-    if (d64) d64[i] = v;
-    if (d32) d32[i] = (float)v;
+    if (dia) {
+      d64[i] = k >= 0 ? dia_value(v) : -0.0;
+      d32[i] = k >= 0 ? dia_value((float)v) : -0.f;
+    } else {
+      if (d64) d64[i] = v;
+      if (d32) d32[i] = (float)v;
+    }
   }
 }
 
@@ -1197,8 +1217,6 @@ struct Quad {
 // flight without holding them in registers.  A register-pipelined pass (two
 // 16-byte groups per thread and array) kept far less in flight and streamed
 // the 256^3 system's vectors at about 4.8 TB/s.
-constexpr int kVecChunkBytes = 8192;  // per array and chunk
-constexpr int kVecBufs = 4;           // chunks in flight
 template <typename V>
 __host__ __device__ constexpr int vec_chunk() { return kVecChunkBytes / (int)sizeof(V); }
 struct VecPipe {
@@ -1216,8 +1234,6 @@ __device__ __forceinline__ void vec_pipe_init(VecPipe& vp, uint64_t* bars, long 
     for (int b = 0; b < kVecBufs; ++b) mbar_init(&bars[b], 1);
   fence_mbar_init();
 }
-template <int NA>
-__host__ __device__ constexpr size_t stream_smem_bytes() { return (size_t)kVecBufs * NA * kVecChunkBytes; }
 
 // f(i, v) for every 16-byte group of W rows at row i of [r0, rv), rv = r0 +
 // W floor((r1 - r0) / W), with v[k] = src[k][i .. i + W - 1] (r0 a multiple
@@ -1287,7 +1303,7 @@ __device__ __forceinline__ bool stream_rows(const V* const (&src)[NA], int64_t r
 // true-residual confirmation.  OUTER = true: the full solve of Section III
 // from the caller's x0 with the confirm/restart step.
 template <typename V, int FMT, bool OUTER>
-__global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) k_cg(CgArgs<V> a) {
+__global__ void __launch_bounds__(block_of(FMT), 1) k_cg(CgArgs<V> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bars[kMaxThreads / 32][kMaxStages];
   __shared__ double red[33];
@@ -1314,12 +1330,14 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
   double* part1 = a.part + G;
   __shared__ uint64_t tbar[2 * kMaxTileStages];
   Pipe pp;
-  pipe_init(pp, bars[threadIdx.x >> 5], gather_stages<V>(), a.timeout_ns);
   TilePipe tp;
-  tile_pipe_init(tp, tbar, a.timeout_ns);
+  if constexpr (FMT == kGather) pipe_init(pp, bars[threadIdx.x >> 5], gather_stages<V>(), a.timeout_ns);
+  if constexpr (FMT == kTiles) tile_pipe_init(tp, tbar, a.timeout_ns);
+  __shared__ DiaTab<V> dtab;
+  if constexpr (is_dia(FMT)) dia_tab_init(dtab, a.D);
   __shared__ uint64_t vbar[kVecBufs];
   VecPipe vp;
-  if constexpr (FMT == kTiles) vec_pipe_init(vp, vbar, a.timeout_ns);
+  if constexpr (FMT == kTiles || is_dia(FMT)) vec_pipe_init(vp, vbar, a.timeout_ns);
   static_assert(FMT != kTiles || stream_smem_bytes<5>() <= sizeof(TileSmem<V>), "vector stream buffers");
   __syncthreads();
   int* err = &a.bar->status;
@@ -1332,7 +1350,8 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
 
   // q = A xin over the CTA's rows, complete (kTiles: across a grid barrier)
   auto full_product = [&](const V* xin) -> bool {
-    product_rows<V, FMT, false>(A, T, s0, s1, l0, l1, xin, q, smem_raw, pp, tp, err);
+    if constexpr (is_dia(FMT)) dia_product<V, FMT == kDiaSym>(dtab, r0, r1, xin, q);
+    else product_rows<V, FMT, false>(A, T, s0, s1, l0, l1, xin, q, smem_raw, pp, tp, err);
     if constexpr (FMT == kTiles) {
       if (!grid_barrier(a.bar, target, a.timeout_ns, &sflag, nbar++)) return false;
       sym_incoming<V>(T, q);
@@ -1406,6 +1425,8 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
           q[row] = qo;
           ppq = fma_(xi, fma_(V(2), direct, dxi), ppq);
         });
+      } else if constexpr (is_dia(FMT)) {
+        ppq = dia_sweep<V, FMT == kDiaSym>(dtab, r0, r1, p, q);
       } else {
         Stage<V>* stages = reinterpret_cast<Stage<V>*>(smem_raw) + (threadIdx.x >> 5) * gather_stages<V>();
         spmv_rows<V, FMT == kPlan, false>(A, s0, s1, l0, l1, p, stages, pp, err, [&](int64_t row, V v, V pr) {
@@ -1469,10 +1490,39 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
             streamed = true;
           }
         }
+        if constexpr (is_dia(FMT) && sizeof(V) == 4) {
+          const V* const src[4] = {p, q, x, r};
+          const bool ok = stream_rows<V, 4>(
+              src, r0, r1, reinterpret_cast<V*>(smem_raw), vp, err,
+              [&](int64_t i, const VT (&v)[4]) {
+                const V* pe = reinterpret_cast<const V*>(&v[0]);
+                const V* qe = reinterpret_cast<const V*>(&v[1]);
+                const V* xe = reinterpret_cast<const V*>(&v[2]);
+                const V* re = reinterpret_cast<const V*>(&v[3]);
+                VT xn, rn;
+                V* xo = reinterpret_cast<V*>(&xn);
+                V* ro = reinterpret_cast<V*>(&rn);
+#pragma unroll
+                for (int j = 0; j < W; ++j) {
+                  xo[j] = fma_(al, pe[j], xe[j]);
+                  ro[j] = fma_(-al, qe[j], re[j]);
+                  prr = fma_(ro[j], ro[j], prr);
+                }
+                *reinterpret_cast<VT*>(x + i) = xn;
+                *reinterpret_cast<VT*>(r + i) = rn;
+              },
+              [&](int64_t i) {
+                x[i] = fma_(al, p[i], x[i]);
+                const V ri = fma_(-al, q[i], r[i]);
+                r[i] = ri;
+                prr = fma_(ri, ri, prr);
+              });
+          if (!ok) return;
+        } else
         // (one 16-byte group per thread at a time in the double-precision
         // tiled solve, whose registers are otherwise taken)
         if (!streamed)
-        rows_vec<V, FMT == kTiles && OUTER && sizeof(V) == 8>(
+        rows_vec<V, (is_dia(FMT) || FMT == kTiles) && OUTER && sizeof(V) == 8>(
             r0, r1,
             [&](int64_t i) {
               VT qv = *reinterpret_cast<const VT*>(q + i);
@@ -1521,8 +1571,8 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
       {
         const V be = (V)beta;
         bool streamed = false;
-        if constexpr (FMT == kTiles) {
-          if (a.stream_vec) {
+        if constexpr (FMT == kTiles || (is_dia(FMT) && sizeof(V) == 4)) {
+          if (is_dia(FMT) || a.stream_vec) {
             const V* const src[2] = {p, r};
             const bool ok = stream_rows<V, 2>(
                 src, r0, r1, reinterpret_cast<V*>(smem_raw), vp, err,
@@ -1624,10 +1674,10 @@ struct PcgArgs {
 // recurrence delta - beta gamma / alpha_old, which cancels near the
 // attainable residual: a non-positive value after the first step of a run
 // ends the run into the confirmation instead of reporting NOT_SPD.
-// Row-gather layouts only (kGather, kPlan): their product needs no barrier
-// of its own.
+// Row-gather and diagonal layouts only (not kTiles): their product needs no
+// barrier of its own.
 template <typename V, int FMT>
-__global__ void __launch_bounds__(kCgThreads, 1) k_pcg(PcgArgs<V> pa) {
+__global__ void __launch_bounds__(block_of(FMT), 1) k_pcg(PcgArgs<V> pa) {
   static_assert(FMT != kTiles, "the tiled symmetric product needs a barrier of its own");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bars[kMaxThreads / 32][kMaxStages];
@@ -1653,10 +1703,21 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_pcg(PcgArgs<V> pa) {
   V* wb[2] = {pa.w0, pa.w1};
   const V* __restrict__ b = a.b;
   Pipe pp;
-  pipe_init(pp, bars[threadIdx.x >> 5], gather_stages<V>(), a.timeout_ns);
+  if constexpr (FMT == kGather) pipe_init(pp, bars[threadIdx.x >> 5], gather_stages<V>(), a.timeout_ns);
+  __shared__ DiaTab<V> dtab;
+  if constexpr (is_dia(FMT)) dia_tab_init(dtab, a.D);
   __syncthreads();
   int* err = &a.bar->status;
-  Stage<V>* stages = reinterpret_cast<Stage<V>*>(smem_raw) + (threadIdx.x >> 5) * gather_stages<V>();
+  // f(row, (A xin)_row[, xin_row]) over the CTA's rows
+  auto product = [&](const V* xin, auto&& f) {
+    if constexpr (is_dia(FMT)) {
+      dia_product<V, FMT == kDiaSym>(dtab, r0, r1, xin, q);
+      for (int64_t row = r0 + threadIdx.x; row < r1; row += blockDim.x) emit_row<V>(f, row, q[row], xin[row]);
+    } else {
+      Stage<V>* stages = reinterpret_cast<Stage<V>*>(smem_raw) + (threadIdx.x >> 5) * gather_stages<V>();
+      spmv_rows<V, FMT == kPlan, false>(A, s0, s1, l0, l1, xin, stages, pp, err, f);
+    }
+  };
   unsigned long long target = 0;
   int nbar = 0, status = kOk, k = 0, restarts = 0, par = 0, cur = 0;
   double gamma = 0.0, delta = 0.0, nb = 0.0, rel_true = 0.0;
@@ -1673,14 +1734,14 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_pcg(PcgArgs<V> pa) {
   };
   for (bool first_run = true;; first_run = false) {
     // r = b - A x; then w = A r with r'r, w'r (and b'b)
-    spmv_rows<V, FMT == kPlan, false>(A, s0, s1, l0, l1, x, stages, pp, err, [&](int64_t row, V v) { q[row] = v; });
+    product(x, [&](int64_t row, V v) { q[row] = v; });
     __syncthreads();
     for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) r[i] = b[i] - q[i];
     if (!grid_barrier(a.bar, target, a.timeout_ns, &sflag, nbar++)) return;
     {
       V pg = V(0), pd = V(0), pb = V(0);
       V* __restrict__ w = wb[cur];
-      spmv_rows<V, FMT == kPlan, false>(A, s0, s1, l0, l1, r, stages, pp, err, [&](int64_t row, V v) {
+      product(r, [&](int64_t row, V v) {
         w[row] = v;
         const V ri = r[row];
         pg = fma_(ri, ri, pg);
@@ -1736,7 +1797,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_pcg(PcgArgs<V> pa) {
         const V* __restrict__ w = wb[cur];
         V* __restrict__ wn = wb[cur ^ 1];
         V pg = V(0), pd = V(0);
-        spmv_rows<V, FMT == kPlan, false>(A, s0, s1, l0, l1, w, stages, pp, err, [&](int64_t row, V qv, V wi) {
+        product(w, [&](int64_t row, V qv, V wi) {
           const V ri = r[row];
           const V zi = first ? qv : fma_(be, zv[row], qv);
           const V si = first ? wi : fma_(be, sv[row], wi);
@@ -1765,7 +1826,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_pcg(PcgArgs<V> pa) {
     }
     {
       // confirm on the true residual; restart the recurrences from it otherwise
-      spmv_rows<V, FMT == kPlan, false>(A, s0, s1, l0, l1, x, stages, pp, err, [&](int64_t row, V v) { q[row] = v; });
+      product(x, [&](int64_t row, V v) { q[row] = v; });
       __syncthreads();
       V ptt = V(0);
       for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
@@ -1805,6 +1866,7 @@ struct RuArgs {
   CgArgs<float> c;        // float operator; x = correction d, r, p, q
   OpDev<double> A64;      // the same layout with double values
   SymDev<double> T64;     // and its tiles (kTiles)
+  DiaDev<double> D64;     // or its diagonals (kDia, kDiaSym)
   double* x64;            // caller's x (in: x0)
   const double* b64;
   double* q64;            // double product scratch
@@ -1824,7 +1886,7 @@ __host__ __device__ constexpr size_t ru_warp_stage_bytes() {
 // TileSmem<float>); each product drains its fills and grid barriers separate
 // them, so no fill of one lands in a stage the other is reading.
 template <int FMT>
-__global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) k_cg_ru(RuArgs ra) {
+__global__ void __launch_bounds__(block_of(FMT), 1) k_cg_ru(RuArgs ra) {
   static_assert(gather_stages<float>() + gather_stages<double>() <= kMaxStages, "mbarrier sets");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bars[kMaxThreads / 32][kMaxStages];
@@ -1852,14 +1914,22 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
   Stage<float>* st32 = reinterpret_cast<Stage<float>*>(wst);
   Stage<double>* st64 = reinterpret_cast<Stage<double>*>(wst);
   Pipe pp32, pp64;
-  pipe_init(pp32, bars[warp], gather_stages<float>(), a.timeout_ns);
-  pipe_init(pp64, bars[warp] + gather_stages<float>(), gather_stages<double>(), a.timeout_ns);
+  if constexpr (FMT == kGather) {
+    pipe_init(pp32, bars[warp], gather_stages<float>(), a.timeout_ns);
+    pipe_init(pp64, bars[warp] + gather_stages<float>(), gather_stages<double>(), a.timeout_ns);
+  }
   __shared__ uint64_t tbar[2 * kMaxTileStages];
   TilePipe tp;
   if constexpr (FMT == kTiles) tile_pipe_init(tp, tbar, a.timeout_ns);
+  __shared__ DiaTab<float> dtab;
+  __shared__ DiaTab<double> dtab64;
+  if constexpr (is_dia(FMT)) {
+    dia_tab_init(dtab, a.D);
+    dia_tab_init(dtab64, ra.D64);
+  }
   __shared__ uint64_t vbar[kVecBufs];
   VecPipe vp;
-  if constexpr (FMT == kTiles) vec_pipe_init(vp, vbar, a.timeout_ns);
+  if constexpr (FMT == kTiles || is_dia(FMT)) vec_pipe_init(vp, vbar, a.timeout_ns);
   static_assert(stream_smem_bytes<5>() <= sizeof(TileSmem<float>), "vector stream buffers");
   __syncthreads();
   int* err = &a.bar->status;
@@ -1884,6 +1954,8 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
                                [&](int64_t row, double qo, double, double, double) { q64[row] = qo; });
       if (!grid_barrier(a.bar, target, a.timeout_ns, &sflag, nbar++)) return false;
       sym_incoming<double>(ra.T64, q64);
+    } else if constexpr (is_dia(FMT)) {
+      dia_product<double, FMT == kDiaSym>(dtab64, r0, r1, x64, q64);
     } else {
       spmv_rows<double, FMT == kPlan, false>(ra.A64, s0, s1, l0, l1, x64, st64, pp64, err,
                                              [&](int64_t row, double v) { q64[row] = v; });
@@ -1943,6 +2015,8 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
           q[row] = qo;
           ppq = fmaf(xi, fmaf(2.f, direct, dxi), ppq);
         });
+      } else if constexpr (is_dia(FMT)) {
+        ppq = dia_sweep<float, FMT == kDiaSym>(dtab, r0, r1, p, q);
       } else {
         spmv_rows<float, FMT == kPlan, false>(a.A, s0, s1, l0, l1, p, st32, pp32, err,
                                               [&](int64_t row, float v, float pr) {
@@ -1994,6 +2068,37 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
           [&](int64_t i) {
             d[i] = fmaf(al, p[i], d[i]);
             const float ri = fmaf(-al, q[i] + a.T.p1[i], r[i]);
+            r[i] = ri;
+            prr = fmaf(ri, ri, prr);
+          });
+      if (!ok) return;
+      const double sr = block_sum((double)prr, red);
+      if (threadIdx.x == 0) part1[c] = sr;
+    } else if (is_dia(FMT)) {
+      float prr = 0.f;
+      const float* const src[4] = {p, q, d, r};
+      const bool ok = stream_rows<float, 4>(
+          src, r0, r1, reinterpret_cast<float*>(smem_raw), vp, err,
+          [&](int64_t i, const float4 (&v)[4]) {
+            const float* pe = reinterpret_cast<const float*>(&v[0]);
+            const float* qe = reinterpret_cast<const float*>(&v[1]);
+            const float* de = reinterpret_cast<const float*>(&v[2]);
+            const float* re = reinterpret_cast<const float*>(&v[3]);
+            float4 dn, rn;
+            float* dno = reinterpret_cast<float*>(&dn);
+            float* rno = reinterpret_cast<float*>(&rn);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              dno[j] = fmaf(al, pe[j], de[j]);
+              rno[j] = fmaf(-al, qe[j], re[j]);
+              prr = fmaf(rno[j], rno[j], prr);
+            }
+            *reinterpret_cast<float4*>(d + i) = dn;
+            *reinterpret_cast<float4*>(r + i) = rn;
+          },
+          [&](int64_t i) {
+            d[i] = fmaf(al, p[i], d[i]);
+            const float ri = fmaf(-al, q[i], r[i]);
             r[i] = ri;
             prr = fmaf(ri, ri, prr);
           });
@@ -2058,7 +2163,7 @@ __global__ void __launch_bounds__(FMT == kTiles ? kTileThreads : kCgThreads, 1) 
     }
     rr = rr_new;
     // C: p = r + beta p
-    if (FMT == kTiles && ra.c.stream_vec) {
+    if (is_dia(FMT) || (FMT == kTiles && ra.c.stream_vec)) {
       const float* const src[2] = {p, r};
       const bool ok = stream_rows<float, 2>(
           src, r0, r1, reinterpret_cast<float*>(smem_raw), vp, err,

@@ -20,8 +20,10 @@ struct Rows {
   std::vector<double> rv;
 };
 
-int validate(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
-             int32_t base, std::string& err) {
+}  // namespace
+
+int validate_input(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
+                   int32_t base, std::string& err) {
   char buf[256];
   if (n < 0 || nnz < 0) { err = "n and nnz must be non-negative"; return kErrInvalid; }
   if (n > 0x7fffffffLL - 64) { err = "n exceeds the int32 index range"; return kErrInvalid; }
@@ -76,6 +78,60 @@ int validate(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const i
   }
   return 0;
 }
+
+bool build_diagonals(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
+                     int32_t base, DiaHost& out) {
+  out = DiaHost();
+  if (n == 0 || nnz == 0) return false;
+  // the distinct offsets (line - index), increasing; lines hold increasing
+  // indices, so one pass over a line walks the list once
+  std::vector<int32_t> off;
+  for (int64_t r = 0; r < n; ++r) {
+    size_t at = 0;
+    for (int64_t k = (int64_t)ptr[r] - base; k < (int64_t)ptr[r + 1] - base; ++k) {
+      const int32_t o = (int32_t)((int64_t)idx[k] - base - r);
+      while (at < off.size() && off[at] < o) ++at;
+      if (at < off.size() && off[at] == o) continue;
+      if (off.size() == (size_t)kMaxDiag) return false;
+      off.insert(off.begin() + at, o);
+    }
+  }
+  if (format == 1 && off[0] != 0) off.insert(off.begin(), 0);  // the kernels take off[0] as the diagonal
+  if (off.size() > (size_t)kMaxDiag || 3 * (long double)nnz < 2 * (long double)off.size() * n) return false;
+  // after a diagonal's values, padding where a mirrored index below 0 leads,
+  // and the rows a segment may run past the last one
+  const int64_t ld = (n + std::max(0, off.back()) + kDiaHalo + 63) & ~int64_t(63);
+  if ((int64_t)off.size() * ld > 0xffffffffLL || n > (int64_t(1) << 28)) return false;  // 32-bit offsets
+  out.ld = ld;
+  out.val.assign(off.size() * (size_t)ld, -0.0);
+  int64_t zero_diag = 0, diag = 0;
+  for (int64_t r = 0; r < n; ++r) {
+    size_t at = 0;
+    for (int64_t k = (int64_t)ptr[r] - base; k < (int64_t)ptr[r + 1] - base; ++k) {
+      const int64_t c = (int64_t)idx[k] - base;
+      const int32_t o = (int32_t)(c - r);
+      while (off[at] != o) ++at;
+      const double v = val[k] == 0.0 ? 0.0 : val[k];
+      if (format == 2)  // line r is column r: row c, offset r - c, on the list reversed
+        out.val[(off.size() - 1 - at) * (size_t)ld + c] = v;
+      else
+        out.val[at * (size_t)ld + r] = v;
+      if (o == 0) {
+        ++diag;
+        if (val[k] == 0.0) ++zero_diag;
+      }
+    }
+  }
+  if (format == 2) {
+    std::reverse(off.begin(), off.end());
+    for (int32_t& o : off) o = -o;
+  }
+  out.nnz_full = format == 1 ? 2 * (nnz - diag) + diag - zero_diag : nnz;
+  out.off = off;
+  return true;
+}
+
+namespace {
 
 // Slices rows into the SELL-32 layout; rows longer than `long_threshold` go
 // to the warp-per-row list when `allow_long`.
@@ -209,7 +265,7 @@ int check_symmetry(int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* id
 
 int build_layout(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                  const double* val, int32_t base, LayoutHost& out, std::string& err) {
-  int rc = validate(format, n, nnz, ptr, idx, val, base, err);
+  int rc = validate_input(format, n, nnz, ptr, idx, val, base, err);
   if (rc) return rc;
   out = LayoutHost();
   out.format = format;

@@ -47,6 +47,23 @@ struct PlanHost {
   std::vector<uint16_t> pl_k;      // slot of U_ij in row i; 0xFFFF = padding
 };
 
+// Diagonal layout.  Entry (i, i + off[k]) lies at val[k * ld + i]: no stored
+// indices.  Symmetric storage keeps the stored upper triangle (off[0] = 0, the
+// rest positive, increasing); full storage every diagonal, increasing.  A
+// position without an entry holds -0.0 (entries that are zero are +0.0).
+// Taken when the matrix has at most kMaxDiag diagonals and at least two
+// thirds of their positions are entries: then a product never reads more
+// bytes than the row-gather layout's 10 or 6 (8 or 4 of value, 2 of index)
+// or the tiles' 6 per entry.
+constexpr int kMaxDiag = 32;
+constexpr int kDiaHalo = 128;  // rows a segment may run past the last one
+struct DiaHost {
+  std::vector<int32_t> off;
+  int64_t ld = 0;           // n + max(off) + kDiaHalo, rounded up to a multiple of 64
+  std::vector<double> val;  // off.size() * ld
+  int64_t nnz_full = 0;     // entries of the full operator
+};
+
 // Tiled symmetric layout.  Rows are split into contiguous ranges, one per CTA
 // of the persistent grid, and each range into tiles of whole slices (up to
 // 15 for double precision, one per consumer warp; up to 30 for single
@@ -146,8 +163,18 @@ struct LayoutHost {
   std::vector<double> urv;
 };
 
-// Validates the input (0- or 1-based) and builds the layout.  Returns 0 or a
-// gbcg_status error code, with a message in `err`.
+// Validates the input (0- or 1-based).  Returns 0 or a gbcg_status error
+// code, with a message in `err`.
+int validate_input(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
+                   int32_t index_base, std::string& err);
+
+// Builds the diagonal layout of a validated input.  Returns false (`out` left
+// empty) when the matrix does not meet its rule.
+bool build_diagonals(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
+                     const double* val, int32_t index_base, DiaHost& out);
+
+// Validates the input and builds the row-gather (or symmetric) layout.
+// Returns 0 or a gbcg_status error code, with a message in `err`.
 int build_layout(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                  const double* val, int32_t index_base, LayoutHost& out, std::string& err);
 
