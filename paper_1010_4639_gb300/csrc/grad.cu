@@ -14,6 +14,7 @@
 // All three are streaming kernels bound by HBM.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 
 #include "../../include/gbcg.h"
@@ -59,34 +60,151 @@ __global__ void __launch_bounds__(256) k_grad_values(int64_t n, const int32_t* _
   }
 }
 
-__global__ void __launch_bounds__(256) k_element_grad(int64_t ne, int m, const int32_t* __restrict__ pos,
-                                                      const double* __restrict__ w, const double* __restrict__ g,
-                                                      double* __restrict__ gc) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < m; ++k) {
-      const int32_t p = pos[e * m + k];
-      if (p >= 0) s = fma(w[e * m + k], g[p], s);
+// The two assembly kernels read a map of one position (or element number) and
+// one weight per contribution, some 24 of them per unknown.  A thread that
+// walks its own contributions from global memory touches a line of its own
+// with every load (a warp's load then takes 32 cycles of L1), waits for each
+// gather before the next, and on k_assemble idles while the one diagonal entry
+// of the warp sums its 24 contributions (on GB300 an FP64 instruction occupies
+// the pipe for 16 cycles whether 1 or 32 lanes take part).  So a block brings
+// a run of contributions, weight and gathered value, into shared memory with
+// contiguous loads, and each output is then summed from there by one thread,
+// in the map's order.  Bounds: the map read once (12 bytes per
+// contribution) and one FP64 FMA each.
+constexpr int kGradThreads = 256;
+constexpr int kStage = 2048;  // contributions staged at a time (16 bytes each)
+constexpr int kPer = kStage / kGradThreads;
+
+// A thread's contributions of a run of `len` starting at tw, tn: every
+// kGradThreads-th.
+struct Contributions {
+  int32_t n[kPer];
+  double w[kPer];
+  __device__ __forceinline__ void load(const int32_t* __restrict__ tn, const double* __restrict__ tw, int len) {
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int j = (int)threadIdx.x + u * kGradThreads;
+      n[u] = -1;
+      w[u] = 0.0;
+      if (j < len) {
+        n[u] = __ldcs(tn + j);
+        w[u] = __ldcs(tw + j);
+      }
     }
-    gc[e] = s;
+  }
+};
+constexpr int kGradBlocks = 6;  // blocks per SM that the stage leaves room for
+
+// gc[e] = sum over k of w[e, k] g[pos[e, k]].  64^3 nodes, full storage (1.5 M
+// elements of 16 pairs, 288 MB of map): 140 us with a thread per element, 97
+// staged, 70 with the next run's map loaded into registers before the sums of
+// the present one start (which the assembly below has no registers for: 124 us
+// without, 160 with).
+// Elements lie an odd number of 16-byte pairs apart, so eight lanes' reads of
+// a step fall into different banks.
+__global__ void __launch_bounds__(kGradThreads, 4) k_element_grad(int64_t ne, int m, int per, uint32_t inv,
+                                                               const int32_t* __restrict__ pos,
+                                                               const double* __restrict__ w,
+                                                               const double* __restrict__ g,
+                                                               double* __restrict__ gc) {
+  extern __shared__ double2 stage[];
+  const int ms = m | 1;
+  const int64_t step = (int64_t)gridDim.x * per;
+  auto elements = [&](int64_t e0) { return (int)(ne - e0 < per ? ne - e0 : per); };
+  Contributions c;
+  int64_t e0 = (int64_t)blockIdx.x * per;
+  if (e0 < ne) c.load(pos + e0 * m, w + e0 * m, elements(e0) * m);
+  for (; e0 < ne; e0 += step) {
+    const int cnt = elements(e0), len = cnt * m;
+    double gv[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) gv[u] = c.n[u] >= 0 ? __ldg(g + c.n[u]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int j = (int)threadIdx.x + u * kGradThreads;
+      const int e = (int)(((uint32_t)j * inv) >> 20);  // j / m
+      // no position: -0.0 * 0.0 leaves the sum as it is
+      if (j < len) stage[e * ms + (j - e * m)] = make_double2(c.n[u] >= 0 ? c.w[u] : -0.0, gv[u]);
+    }
+    __syncthreads();
+    if (e0 + step < ne) c.load(pos + (e0 + step) * m, w + (e0 + step) * m, elements(e0 + step) * m);
+    for (int e = threadIdx.x; e < cnt; e += kGradThreads) {
+      double s = 0.0;
+#pragma unroll 4
+      for (int k = 0; k < m; ++k) {
+        const double2 t = stage[e * ms + k];
+        s = fma(t.x, t.y, s);
+      }
+      gc[e0 + e] = s;
+    }
+    __syncthreads();
   }
 }
 
-__global__ void __launch_bounds__(256) k_assemble(int64_t nnz, const int64_t* __restrict__ tptr,
-                                                  const int32_t* __restrict__ telem, const double* __restrict__ tw,
-                                                  const double* __restrict__ coef, double* __restrict__ val) {
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
+// val[p] = sum over k in [tptr[p], tptr[p + 1]) of tw[k] coef[telem[k]], 256
+// positions per block.  The block's threads take its positions in order of
+// their numbers of contributions, so that the 32 sums of a warp are about
+// equally long.  64^3 nodes, full storage (3.5 M positions, 23 M
+// contributions): 190 us with a thread per position, 124 so.
+__global__ void __launch_bounds__(kGradThreads) k_assemble(int64_t nnz, const int64_t* __restrict__ tptr,
+                                                           const int32_t* __restrict__ telem,
+                                                           const double* __restrict__ tw,
+                                                           const double* __restrict__ coef, double* __restrict__ val) {
+  constexpr int kBins = 32;
+  __shared__ double2 stage[kStage];
+  __shared__ int64_t ptr[kGradThreads + 1];
+  __shared__ int bin[kBins];
+  __shared__ uint8_t order[kGradThreads];
+  const int t = threadIdx.x;
+  for (int64_t p0 = (int64_t)blockIdx.x * kGradThreads; p0 < nnz; p0 += (int64_t)gridDim.x * kGradThreads) {
+    const int cnt = (int)(nnz - p0 < kGradThreads ? nnz - p0 : kGradThreads);
+    for (int i = t; i <= cnt; i += kGradThreads) ptr[i] = tptr[p0 + i];
+    if (t < kBins) bin[t] = 0;
+    __syncthreads();
+    // a counting sort by number of contributions (ties in any order: it only
+    // decides which thread sums which position)
+    const int64_t n0 = t < cnt ? ptr[t + 1] - ptr[t] : 0;
+    const int b = n0 < kBins ? (int)n0 : kBins - 1;
+    const int rank = t < cnt ? atomicAdd(&bin[b], 1) : 0;
+    __syncthreads();
+    if (t < kBins) {
+      const int own = bin[t];
+      int sum = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, sum, o);
+        if (t >= o) sum += up;
+      }
+      bin[t] = sum - own;
+    }
+    __syncthreads();
+    if (t < cnt) order[bin[b] + rank] = (uint8_t)t;
+    __syncthreads();
+    const int mine = t < cnt ? order[t] : -1;
+    const int64_t k0 = mine >= 0 ? ptr[mine] : 0, k1 = mine >= 0 ? ptr[mine + 1] : 0;
     double s = 0.0;
-    for (int64_t k = tptr[p]; k < tptr[p + 1]; ++k) s = fma(tw[k], coef[telem[k]], s);
-    val[p] = s;
+    for (int64_t c0 = ptr[0], end = ptr[cnt]; c0 < end; c0 += kStage) {
+      const int len = (int)(end - c0 < kStage ? end - c0 : kStage);
+#pragma unroll 4
+      for (int j = t; j < len; j += kGradThreads)
+        stage[j] = make_double2(__ldcs(tw + c0 + j), __ldg(coef + __ldcs(telem + c0 + j)));
+      __syncthreads();
+      const int a = (int)(k0 < c0 ? 0 : k0 - c0 < len ? k0 - c0 : len);
+      const int z = (int)(k1 < c0 ? 0 : k1 - c0 < len ? k1 - c0 : len);
+#pragma unroll 2
+      for (int j = a; j < z; ++j) s = fma(stage[j].x, stage[j].y, s);
+      __syncthreads();
+    }
+    if (mine >= 0) val[p0 + mine] = s;
+    __syncthreads();  // ptr, bin and order are rewritten
   }
 }
 
-int grid_for(int64_t items, int per_block) {
+int grid_for(int64_t items, int per_block, int blocks_per_sm = 8) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t want = (items + per_block - 1) / per_block;
-  const int64_t cap = (int64_t)sms * 8;
+  const int64_t cap = (int64_t)sms * blocks_per_sm;
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
@@ -126,7 +244,12 @@ int gbcg_element_grad(int64_t ne, int32_t m, const int32_t* pos, const double* w
   if (ne < 0 || m < 0 || m > 64) return fail(GBCG_ERR_INVALID, "ne must be >= 0 and m in [0, 64]");
   if (ne == 0) return GBCG_OK;
   if (!grad_coef || (m > 0 && (!pos || !w || !grad))) return fail(GBCG_ERR_INVALID, "null argument");
-  k_element_grad<<<grid_for(ne, 256), 256, 0, (cudaStream_t)stream>>>(ne, m, pos, w, grad, grad_coef);
+  // elements per block: what the stage holds, at most one per thread; j / m =
+  // (j inv) >> 20 for j < 2^20 / m
+  const int per = m > 0 ? std::min(kGradThreads, kStage / (m | 1)) : kGradThreads;
+  const uint32_t inv = m > 0 ? ((1u << 20) + m - 1) / m : 0;
+  k_element_grad<<<grid_for(ne, per, 4), kGradThreads, sizeof(double2) * per * (m | 1), (cudaStream_t)stream>>>(
+      ne, m, per, inv, pos, w, grad, grad_coef);
   return launched("k_element_grad");
 }
 
@@ -136,7 +259,7 @@ int gbcg_assemble(int64_t nnz, const int64_t* tptr, const int32_t* telem, const 
   if (nnz < 0) return fail(GBCG_ERR_INVALID, "nnz must be >= 0");
   if (nnz == 0) return GBCG_OK;
   if (!tptr || !val || !telem || !tw || !coef) return fail(GBCG_ERR_INVALID, "null argument");
-  k_assemble<<<grid_for(nnz, 256), 256, 0, (cudaStream_t)stream>>>(nnz, tptr, telem, tw, coef, val);
+  k_assemble<<<grid_for(nnz, kGradThreads, kGradBlocks), kGradThreads, 0, (cudaStream_t)stream>>>(nnz, tptr, telem, tw, coef, val);
   return launched("k_assemble");
 }
 
