@@ -34,10 +34,17 @@
 #include <vector>
 
 #include "../../include/gbcg.h"
+#include "fp64.cuh"
 
 namespace gbcg {
 void set_last_error(const std::string& m);
 }
+
+using gbcg::quick_div;
+using gbcg::quick_double;
+using gbcg::quick_finite;
+using gbcg::quick_positive;
+using gbcg::SqrtTest;
 
 namespace {
 
@@ -147,8 +154,12 @@ __device__ __forceinline__ int ld_dsmem_s32(const int* local, unsigned rank) {
   return v;
 }
 
+constexpr int kSumWarps = 4;  // warps that add a CTA's partial sums
 struct Red {
-  double warp[kMaxWarps][2 * kRhs];
+  // per-thread partial sums of one set of eight, value j of thread t at
+  // j * (NT + 8) + t (NT threads of VW values: 16 bytes each)
+  alignas(16) unsigned char buf[kMaxWarps * 32 * 16 + 8 * 16];
+  double part[kSumWarps][2 * kRhs];
   double cta[2][2 * kRhs];
   double sum[2 * kRhs];
 };
@@ -157,48 +168,74 @@ struct Red {
 // right-hand side k, every other thread only reads.
 struct St {
   double rr[kRhs], nr0[kRhs], nb[kRhs], nr[kRhs], alpha[kRhs], beta[kRhs], rel[kRhs], itol[kRhs], rmax[kRhs];
+  SqrtTest at_tol[kRhs], at_delta[kRhs];  // r'r against the pass's target, and (reliable updates) the next update's
   int used[kRhs], outer[kRhs], status[kRhs], kin[kRhs], bd[kRhs];
   unsigned fin, oact, iact, zero;
   int maxit, products, outers;
 };
 
 // Cluster-wide sums of NS x 8 values.  v[s][j] is this thread's partial of
-// sum (s, c*VW + j), c = lane % (8/VW) the thread's group of right-hand
-// sides.  Fixed order everywhere: lanes by xor tree, warps in index order,
-// CTAs in rank order.  The result for sum t = s*8 + k is returned on thread
+// sum (s, c*VW + j), c = t % (8/VW) the thread's group of right-hand sides.
+// Fixed order everywhere.  The result for sum t = s*8 + k is returned on thread
 // t (t < NS*8); every CTA of the cluster computes identical values.
-template <int VW, int NS>
-__device__ __forceinline__ double cluster_reduce(double (&v)[NS][VW], Red& red, int& par, unsigned C) {
-  constexpr int CH = kRhs / VW;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+//
+// A shuffle tree per warp and value would issue 16 FP64 additions in each of
+// 16 warps: 4 100 cycles of the SM's FP64 pipe per set of eight sums (fp64.cuh),
+// twice per iteration, which was a third of an iteration.  Instead the partial
+// sums go to shared memory, where lane (k, q) of four warps adds those of
+// right-hand side k whose thread is q modulo 16 groups (consecutive lanes in
+// consecutive banks), and the lanes, warps and CTAs are added by short trees:
+// 1 400 cycles.
+template <int NT, int NS, typename T, int VW>
+__device__ __forceinline__ double cluster_reduce(const T (&v)[NS][VW], Red& red, int& par, unsigned C) {
+  constexpr int CH = kRhs / VW, Q = 4 * kSumWarps;
+  constexpr int pitch = NT + 8;  // the four or two values of a thread fall into different banks
+  static_assert((size_t)VW * pitch * sizeof(T) <= sizeof(red.buf), "partial sums");
+  static_assert(NT / CH % Q == 0, "every lane adds the same number");
+  T* buf = reinterpret_cast<T*>(red.buf);
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, k = lane & 7;
 #pragma unroll
-  for (int s = 0; s < NS; ++s)
+  for (int s = 0; s < NS; ++s) {
+    if (s > 0) __syncthreads();
 #pragma unroll
-    for (int j = 0; j < VW; ++j) {
-      double t = v[s][j];
+    for (int j = 0; j < VW; ++j) buf[j * pitch + t] = v[s][j];
+    __syncthreads();
+    if (w < kSumWarps) {
+      const T* b = buf + (k % VW) * pitch + k / VW + CH * (4 * w + (lane >> 3));
+      double x = quick_double(b[0]);
 #pragma unroll
-      for (int o = CH; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      v[s][j] = t;
+      for (int i = 1; i < NT / CH / Q; ++i) x += quick_double(b[CH * Q * i]);
+      x += __shfl_xor_sync(0xffffffffu, x, 8);
+      x += __shfl_xor_sync(0xffffffffu, x, 16);
+      if (lane < kRhs) red.part[w][s * kRhs + lane] = x;
     }
-  if (lane < CH) {
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-#pragma unroll
-      for (int j = 0; j < VW; ++j) red.warp[w][s * kRhs + lane * VW + j] = v[s][j];
   }
   __syncthreads();
-  const int nw = blockDim.x >> 5;
-  if (threadIdx.x < NS * kRhs) {
-    double t = 0.0;
-    for (int i = 0; i < nw; ++i) t += red.warp[i][threadIdx.x];
-    red.cta[par][threadIdx.x] = t;
-  }
+  if (t < NS * kRhs)
+    red.cta[par][t] = (red.part[0][t] + red.part[1][t]) + (red.part[2][t] + red.part[3][t]);
   cluster_sync();
-  double s = 0.0;
-  if (threadIdx.x < NS * kRhs)
-    for (unsigned c = 0; c < C; ++c) s += ld_dsmem_f64(&red.cta[par][threadIdx.x], c);
+  double r = 0.0;
+  if (w == 0) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      // lane (k, q) adds CTAs q, q + 4, ...; then the four lanes of k
+      double x = 0.0;
+      for (unsigned c = lane >> 3; c < C; c += 4) {
+        const double y = ld_dsmem_f64(&red.cta[par][s * kRhs + k], c);
+        x = c < 4 ? y : x + y;
+      }
+      if (C > 1) x += __shfl_xor_sync(0xffffffffu, x, 8);
+      if (C > 2) x += __shfl_xor_sync(0xffffffffu, x, 16);
+      if ((lane >> 3) == s) r = x;
+    }
+    if (C == 1) {  // lanes 0 .. 7 hold the only CTA's sums
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+        if ((lane >> 3) == s) r = red.cta[par][s * kRhs + k];
+    }
+  }
   par ^= 1;
-  return s;
+  return r;
 }
 
 template <typename VT, typename V>
@@ -370,10 +407,10 @@ __device__ __forceinline__ bool group_sync(const BArgs& a, Group& g, int* s_flag
 
 // Sums over the whole group (see cluster_reduce): the cluster's sums, then
 // for G > 1 the parts' sums in part order, read from global memory.
-template <int VW, int NS>
-__device__ __forceinline__ double group_reduce(const BArgs& a, double (&v)[NS][VW], Red& red, int& par, Group& g,
+template <int NT, int NS, typename T, int VW>
+__device__ __forceinline__ double group_reduce(const BArgs& a, const T (&v)[NS][VW], Red& red, int& par, Group& g,
                                                int* s_flag, bool& ok) {
-  double s = cluster_reduce<VW, NS>(v, red, par, g.C);
+  double s = cluster_reduce<NT, NS>(v, red, par, g.C);
   if (g.G == 1) return s;
   double* slot = g.part + g.gpar * (kMaxGroup * 2 * kRhs);
   if (g.cr == 0 && threadIdx.x < NS * kRhs) slot[g.p * 2 * kRhs + threadIdx.x] = s;
@@ -383,6 +420,12 @@ __device__ __forceinline__ double group_reduce(const BArgs& a, double (&v)[NS][V
   if (threadIdx.x < NS * kRhs)
     for (int q = 0; q < g.G; ++q) s += __ldcg(slot + q * 2 * kRhs + threadIdx.x);
   return s;
+}
+
+template <int NT, typename T, int VW>
+__device__ __forceinline__ double group_reduce1(const BArgs& a, const T (&v)[VW], Red& red, int& par, Group& g,
+                                                int* s_flag, bool& ok) {
+  return group_reduce<NT, 1>(a, reinterpret_cast<const T(&)[1][VW]>(v), red, par, g, s_flag, ok);
 }
 
 // One instance, all right-hand sides, on this cluster's share of its rows.
@@ -430,7 +473,7 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
     {
       double v[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
       outer_residual(a, r0, r1, v);
-      const double s = group_reduce<2, 2>(a, v, red, par, g, s_flag, ok);
+      const double s = group_reduce<NT, 2>(a, v, red, par, g, s_flag, ok);
       if (!ok) return false;
       if (t >= kRhs && t < 2 * kRhs) red.sum[t] = s;
       __syncthreads();
@@ -509,16 +552,14 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
         reinterpret_cast<VT*>(P)[e] = rv;
         reinterpret_cast<VT*>(D)[e] = VT{};
       }
-      double v[1][VW];
-#pragma unroll
-      for (int j = 0; j < VW; ++j) v[0][j] = (double)pr[j];
-      const double s = group_reduce<VW, 1>(a, v, red, par, g, s_flag, ok);  // also publishes P
+      const double s = group_reduce1<NT>(a, pr, red, par, g, s_flag, ok);  // also publishes P
       if (!ok) return false;
       if (t < 32) {
         bool go = false;
         if (t < kRhs && ((oact >> t) & 1u)) {
           st.rr[t] = s;
           st.nr0[t] = sqrt(s);
+          st.at_tol[t].set(st.itol[t] * st.nr0[t]);
           st.kin[t] = 0;
           st.bd[t] = 0;
           go = st.nr0[t] > 0.0 && !(sqrt(s) <= st.itol[t] * st.nr0[t]) && st.used[t] < st.maxit;
@@ -532,7 +573,6 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
     while (st.iact) {
       // q = A p, p'q
       {
-        double v[1][VW];
         V pq[VW];
 #pragma unroll
         for (int j = 0; j < VW; ++j) pq[j] = V(0);
@@ -545,17 +585,15 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
 #pragma unroll
           for (int j = 0; j < VW; ++j) pq[j] = pe[j] * qe[j] + pq[j];
         });
-#pragma unroll
-        for (int j = 0; j < VW; ++j) v[0][j] = (double)pq[j];
-        const double s = group_reduce<VW, 1>(a, v, red, par, g, s_flag, ok);
+        const double s = group_reduce1<NT>(a, pq, red, par, g, s_flag, ok);
         if (!ok) return false;
         if (t < kRhs) {
           double al = 0.0;
           if ((st.iact >> t) & 1u) {
-            if (!isfinite(s) || !(s > 0.0))
+            if (!quick_finite(s) || !quick_positive(s))
               st.bd[t] = 1;
             else
-              al = st.rr[t] / s;
+              al = quick_div<V>(st.rr[t], s);
           }
           st.alpha[t] = al;
         }
@@ -587,10 +625,7 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
           reinterpret_cast<VT*>(D)[e] = dv;
           reinterpret_cast<VT*>(R)[e] = rv;
         }
-        double v[1][VW];
-#pragma unroll
-        for (int j = 0; j < VW; ++j) v[0][j] = (double)pr[j];
-        const double s = group_reduce<VW, 1>(a, v, red, par, g, s_flag, ok);
+        const double s = group_reduce1<NT>(a, pr, red, par, g, s_flag, ok);
         if (!ok) return false;
         if (t < 32) {
           bool go = false;
@@ -600,10 +635,10 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
             } else {
               st.kin[t] += 1;
               st.used[t] += 1;
-              if (sqrt(s) <= st.itol[t] * st.nr0[t]) {
+              if (st.at_tol[t].below(s, [&] { return sqrt(s) <= st.itol[t] * st.nr0[t]; })) {
                 st.beta[t] = 0.0;
               } else {
-                st.beta[t] = s / st.rr[t];
+                st.beta[t] = quick_div<V>(s, st.rr[t]);
                 st.rr[t] = s;
                 go = st.used[t] < st.maxit;
               }
@@ -745,14 +780,17 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
     if (!group_sync(a, g, s_flag)) return false;  // x of every CTA before the product
     double v[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
     outer_residual(a, r0, r1, v);
-    const double s = group_reduce<2, 2>(a, v, red, par, g, s_flag, ok);
+    const double s = group_reduce<NT, 2>(a, v, red, par, g, s_flag, ok);
     if (!ok) return false;
     if (t >= kRhs && t < 2 * kRhs) red.sum[t] = s;
     __syncthreads();
     if (t < 32) {
       bool zero = false, done = false;
       if (t < kRhs && !((st.fin >> t) & 1u)) {
-        if (first) st.nb[t] = sqrt(red.sum[kRhs + t]);
+        if (first) {
+          st.nb[t] = sqrt(red.sum[kRhs + t]);
+          st.at_tol[t].set(a.tol * st.nb[t]);
+        }
         const double nb = st.nb[t];
         if (nb == 0.0) {
           zero = true;
@@ -806,14 +844,12 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
         }
         reinterpret_cast<VT*>(R)[e] = rv;
       }
-      double w[1][VW];
-#pragma unroll
-      for (int j = 0; j < VW; ++j) w[0][j] = (double)pr[j];
-      const double s2 = group_reduce<VW, 1>(a, w, red, par, g, s_flag, ok);
+      const double s2 = group_reduce1<NT>(a, pr, red, par, g, s_flag, ok);
       if (!ok) return false;
       if (t < kRhs) {
         st.nr[t] = s2;  // r'r of the replaced residual
         st.rmax[t] = sqrt(s2);
+        st.at_delta[t].set(a.inner_tol * st.rmax[t]);
       }
       __syncthreads();
     }
@@ -838,23 +874,21 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
         for (int j = 0; j < VW; ++j) pq[j] = fmaf(pe[j], qe[j], pq[j]);
       });
       double v[1][VW];
-#pragma unroll
-      for (int j = 0; j < VW; ++j) v[0][j] = (double)pq[j];
-      const double s = group_reduce<VW, 1>(a, v, red, par, g, s_flag, ok);
+      const double s = group_reduce1<NT>(a, pq, red, par, g, s_flag, ok);
       if (!ok) return false;
       if (t < 32) {
         bool stop = false;
         if (t < kRhs) {
           double al = 0.0;
           if (!((st.fin >> t) & 1u)) {
-            if (!isfinite(s)) {
+            if (!quick_finite(s)) {
               st.status[t] = kNonfinite;
               stop = true;
-            } else if (!(s > 0.0)) {
+            } else if (!quick_positive(s)) {
               st.status[t] = kNotSpd;
               stop = true;
             } else {
-              al = st.rr[t] / s;
+              al = quick_div<float>(st.rr[t], s);
             }
           }
           st.alpha[t] = al;
@@ -887,18 +921,16 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
         reinterpret_cast<VT*>(D)[e] = dv;
         reinterpret_cast<VT*>(R)[e] = rv;
       }
-      double v[1][VW];
-#pragma unroll
-      for (int j = 0; j < VW; ++j) v[0][j] = (double)pr[j];
-      const double s = group_reduce<VW, 1>(a, v, red, par, g, s_flag, ok);
+      const double s = group_reduce1<NT>(a, pr, red, par, g, s_flag, ok);
       if (!ok) return false;
       if (t < 32) {
         bool need = false;
         if (t < kRhs && !((st.fin >> t) & 1u) && st.alpha[t] != 0.0) {
           st.used[t] += 1;
           st.nr[t] = s;
-          const double nr = sqrt(s);
-          need = nr < a.inner_tol * st.rmax[t] || nr <= a.tol * st.nb[t] || st.used[t] >= st.maxit;
+          need = st.used[t] >= st.maxit ||
+                 st.at_delta[t].below(s, [&] { return sqrt(s) < a.inner_tol * st.rmax[t]; }) ||
+                 st.at_tol[t].below(s, [&] { return sqrt(s) <= a.tol * st.nb[t]; });
         } else if (t < kRhs) {
           st.nr[t] = st.rr[t];
         }
@@ -920,7 +952,7 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
     {
       if (t < kRhs) {
         const bool live = !((st.fin >> t) & 1u);
-        st.beta[t] = live ? st.nr[t] / st.rr[t] : 0.0;
+        st.beta[t] = live ? quick_div<float>(st.nr[t], st.rr[t]) : 0.0;
         if (live) st.rr[t] = st.nr[t];
       }
       __syncthreads();

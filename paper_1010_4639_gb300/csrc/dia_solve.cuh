@@ -14,6 +14,7 @@
 //
 // The arithmetic is that of k_cg and k_cg_ru (kernels.cuh), step by step.
 #pragma once
+#include "fp64.cuh"
 #include "kernels.cuh"
 
 namespace gbcg {
@@ -53,8 +54,7 @@ struct GridSum {
 // step's scalars).  False, uniformly within the CTA, when a wait ran out or
 // another CTA failed.
 //
-// An FP64 addition takes 64 cycles on GB300 and occupies its SM
-// sub-partition's FP64 pipe all that time, useful lanes or not, so the CTA's
+// FP64 additions are slow (fp64.cuh), useful lanes or not, so the CTA's
 // partial sums go through shared memory and are added by one warp (four when
 // there are many) instead of a shuffle tree in every warp.  Measured with 152
 // CTAs: an arrival at one counter that a warp per CTA polls costs 2 600
@@ -141,23 +141,6 @@ __device__ __forceinline__ bool chip_barrier(GridSum& g) {
   return grid_barrier(&g.sync->bar, g.target, g.timeout_ns, g.ok, g.sums);
 }
 
-// a / b, accurate to the rounding of V.  FP64 division takes 650 cycles here
-// and sits between a grid sum and the next phase of every CTA.  A reciprocal
-// estimate with one Newton step gives a quotient within 2^-38, enough for a
-// single-precision result; one correction by the quotient's residual makes it
-// a double-precision one.
-template <typename V>
-__device__ __forceinline__ double chip_div(double a, double b) {
-  const int ea = (__double2hiint(a) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
-  if (ea < 128 || ea > 1918 || eb < 128 || eb > 1918) return a / b;  // near the ends of the range, 0, inf, NaN
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
-  r = fma(r, fma(-b, r, 1.0), r);
-  const double q = a * r;
-  return sizeof(V) == 4 ? q : fma(fma(-b, q, a), r, q);
-}
-__device__ __forceinline__ bool chip_finite(double s) { return ((unsigned)__double2hiint(s) & 0x7ff00000u) != 0x7ff00000u; }
-
 // chip_sum of one value per thread whose sum is expected within 2^-13 .. 2^20
 // of `prev` (the same sum an iteration earlier), without a memory fence: it
 // orders nothing but the sum itself.  Each CTA adds its partial sum to two
@@ -242,26 +225,6 @@ __device__ __forceinline__ bool chip_sum_fast(GridSum& g, double v, double prev,
   if (*g.ok != 2) return *g.ok != 0;
   return chip_sum<1>(g, v1, f);
 }
-
-// Tests sqrt(s) against a bound c without the square root (690 cycles): s is
-// compared, as an integer, with c^2 a little enlarged and reduced; only in
-// between does the exact test run.
-struct SqrtTest {
-  long long lo = 0, hi = 0x7ff0000000000000ll;  // undecided everywhere
-  __device__ __forceinline__ void set(double c) {
-    const double c2 = c * c;
-    if (c2 > 1e-290 && c2 < 1e290) {
-      lo = __double_as_longlong(c2 * (1.0 - 1e-12));
-      hi = __double_as_longlong(c2 * (1.0 + 1e-12));
-    }
-  }
-  // s >= 0 and finite; exact() decides in between
-  template <class X>
-  __device__ __forceinline__ bool below(double s, X&& exact) const {
-    const long long b = __double_as_longlong(s);
-    return b < lo ? true : b > hi ? false : exact();
-  }
-};
 
 // What a solve does around its iterations: the double-precision solve from
 // x0 with true-residual confirmation and restarts; the single-precision inner
@@ -463,11 +426,11 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
           sq[i] = q;
           ppq = dia_fma(sp[i], q, ppq);
         });
-        v[0] = (double)ppq;
+        v[0] = quick_double(ppq);
       }
       if (!chip_sum_fast(g, v[0], pq, [&](const double (&s)[1]) {
-            sc.code = !chip_finite(s[0]) ? kNonfinite : __double_as_longlong(s[0]) <= 0 ? kNotSpd : kOk;
-            sc.alpha = chip_div<V>(rr, s[0]);
+            sc.code = !quick_finite(s[0]) ? kNonfinite : !quick_positive(s[0]) ? kNotSpd : kOk;
+            sc.alpha = quick_div<V>(rr, s[0]);
           }))
         return;
       pq = g.out[0];
@@ -485,13 +448,13 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
           sr[i] = ri;
           prr = dia_fma(ri, ri, prr);
         }
-        v[0] = (double)prr;
+        v[0] = quick_double(prr);
       }
       // kSolveRu: an update comes first when the recurrence residual has fallen
       // by delta, has reached tol, or the iteration bound is met
       if (!chip_sum_fast(g, v[0], rr, [&](const double (&s)[1]) {
             const double z = s[0];
-            if (!chip_finite(z)) {
+            if (!quick_finite(z)) {
               sc.code = 2;
             } else if constexpr (KIND == kSolveRu) {
               const bool fell = at_delta.below(z, [&] { return sqrt(z) < a.delta * rmax; });
@@ -499,7 +462,7 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
             } else {
               sc.code = at_tol.below(z, [&] { return sqrt(z) / nb <= a.tol; }) ? 1 : 0;
             }
-            sc.beta = chip_div<V>(z, rr);
+            sc.beta = quick_div<V>(z, rr);
           }))
         return;
       ++k;
