@@ -35,6 +35,7 @@
 
 #include "../../include/gbcg.h"
 #include "fp64.cuh"
+#include "layout.h"
 
 namespace gbcg {
 void set_last_error(const std::string& m);
@@ -82,6 +83,15 @@ struct V16<double> {
   static constexpr int W = 2;
 };
 
+// An instance whose matrix has few diagonals (layout.h, DiaHost; full
+// storage): value k of local row i at val[base + k * ld + i], its column
+// i + off[k].  K = 0: the instance stays in CSR.
+struct BDia {
+  int64_t base;
+  int32_t ld, K;
+  int32_t off[gbcg::kMaxDiag];
+};
+
 // Everything a launch reads, kept in device memory so that a captured graph
 // serves every solve (the host rewrites this block before each launch).
 struct BArgs {
@@ -90,6 +100,8 @@ struct BArgs {
   const int32_t* idx;       // global column of every entry
   const double* val64;
   const float* val32;
+  const BDia* dia;          // per instance
+  const float* dia32;
   const int32_t* slot_inst; // queue slot -> instance
   const int32_t* slot_part; // queue slot -> part of a multi-cluster group (0 .. G-1)
   const int8_t* grp;        // clusters per instance (G)
@@ -306,6 +318,46 @@ __device__ __forceinline__ void product_rpw(int rpw, const int32_t* ptr, const i
   }
 }
 
+// The same product by diagonals (single precision), one right-hand-side group
+// of a row per thread: the loads of C diagonals are all in flight at once and
+// contiguous over the warp, where a CSR row waits for its offsets, its columns
+// and then its gathers, entry by entry.  Columns outside the instance are
+// clamped into it (the value there is padding, -0.0).
+template <class Emit>
+__device__ __forceinline__ void product_dia(const BDia& D, const float* __restrict__ val, const float* x,
+                                            int64_t row0, int nI, int64_t r0, int64_t r1, Emit&& emit) {
+  using V = float;
+  using VT = float4;
+  constexpr int CH = 2, C = 4;
+  const int c = threadIdx.x % CH, K = D.K, ld = D.ld;
+  const VT* xi = reinterpret_cast<const VT*>(x) + row0 * CH + c;
+  const V* __restrict__ vi = val + D.base;
+  const int lane = threadIdx.x & 31, lo = D.off[0], hi = D.off[K - 1];
+  for (int i = (int)(r0 - row0) + threadIdx.x / CH, z = (int)(r1 - row0); i < z; i += blockDim.x / CH) {
+    VT acc{};
+    const int first = i - lane / CH;  // of the warp
+    if (first + lo >= 0 && first + 32 / CH - 1 + hi < nI) {
+      for (int kb = 0; kb < K; kb += C) {
+        V v[C];
+        VT xv[C];
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+          const int k = min(kb + j, K - 1);
+          v[j] = __ldg(vi + (uint32_t)(k * ld + i));
+          xv[j] = xi[(i + D.off[k]) * CH];
+        }
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+          if (kb + j < K) acc = vfma(v[j], xv[j], acc);
+      }
+    } else {
+      for (int k = 0; k < K; ++k)
+        acc = vfma(__ldg(vi + (uint32_t)(k * ld + i)), xi[min(max(i + D.off[k], 0), nI - 1) * CH], acc);
+    }
+    emit(row0 + i, c, acc);
+  }
+}
+
 // Outer residual R64 = B - A64 X (caller layout of B and X, nrhs columns),
 // eight lanes per row in pairs of right-hand sides; partial sums of r'r and
 // b'b per right-hand side.
@@ -431,7 +483,8 @@ __device__ __forceinline__ double group_reduce1(const BArgs& a, const T (&v)[VW]
 // One instance, all right-hand sides, on this cluster's share of its rows.
 // Returns false when a group wait failed (the instance is abandoned).
 template <typename V, int NT>
-__device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St& st, int& par, int* s_flag) {
+__device__ bool solve_instance(const BArgs& a, const BDia& dia, int inst, Group& g, Red& red, St& st, int& par,
+                               int* s_flag) {
   using VT = typename V16<V>::T;
   constexpr int VW = V16<V>::W, CH = kRhs / VW;
   const int t = threadIdx.x;
@@ -576,7 +629,7 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
         V pq[VW];
 #pragma unroll
         for (int j = 0; j < VW; ++j) pq[j] = V(0);
-        product_rpw<V>(rp, a.ptr, a.idx, AV, P, r0, r1, [&](int64_t row, int c, VT acc) {
+        auto emit = [&](int64_t row, int c, VT acc) {
           const int64_t e = row * CH + c;
           reinterpret_cast<VT*>(Q)[e] = acc;
           const VT pv = reinterpret_cast<const VT*>(P)[e];
@@ -584,7 +637,14 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
           const V* qe = reinterpret_cast<const V*>(&acc);
 #pragma unroll
           for (int j = 0; j < VW; ++j) pq[j] = pe[j] * qe[j] + pq[j];
-        });
+        };
+        bool done = false;
+        if constexpr (sizeof(V) == 4)
+          if (dia.K > 0) {
+            product_dia(dia, a.dia32, P, row0, (int)nI, r0, r1, emit);
+            done = true;
+          }
+        if (!done) product_rpw<V>(rp, a.ptr, a.idx, AV, P, r0, r1, emit);
         const double s = group_reduce1<NT>(a, pq, red, par, g, s_flag, ok);
         if (!ok) return false;
         if (t < kRhs) {
@@ -723,7 +783,8 @@ __device__ bool solve_instance(const BArgs& a, int inst, Group& g, Red& red, St&
 // directions are kept.  An update serves every right-hand side at once (an
 // update is valid at any time).  outer counts the updates.
 template <int NT>
-__device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, St& st, int& par, int* s_flag) {
+__device__ bool solve_instance_ru(const BArgs& a, const BDia& dia, int inst, Group& g, Red& red, St& st, int& par,
+                                  int* s_flag) {
   using VT = float4;
   constexpr int VW = 4, CH = 2;
   const int t = threadIdx.x;
@@ -864,7 +925,7 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
     // q = A32 p, p'q
     {
       float pq[VW] = {0.f, 0.f, 0.f, 0.f};
-      product_rpw<float>(rp, a.ptr, a.idx, a.val32, P, r0, r1, [&](int64_t row, int c, VT acc) {
+      auto emit = [&](int64_t row, int c, VT acc) {
         const int64_t e = row * CH + c;
         reinterpret_cast<VT*>(Q)[e] = acc;
         const VT pv = reinterpret_cast<const VT*>(P)[e];
@@ -872,7 +933,9 @@ __device__ bool solve_instance_ru(const BArgs& a, int inst, Group& g, Red& red, 
         const float* qe = reinterpret_cast<const float*>(&acc);
 #pragma unroll
         for (int j = 0; j < VW; ++j) pq[j] = fmaf(pe[j], qe[j], pq[j]);
-      });
+      };
+      if (dia.K > 0) product_dia(dia, a.dia32, P, row0, (int)nI, r0, r1, emit);
+      else product_rpw<float>(rp, a.ptr, a.idx, a.val32, P, r0, r1, emit);
       double v[1][VW];
       const double s = group_reduce1<NT>(a, pq, red, par, g, s_flag, ok);
       if (!ok) return false;
@@ -987,6 +1050,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_bcg(const BArgs* __restrict__
   __shared__ St st;
   __shared__ int s_next, s_flag;
   __shared__ Group g;
+  __shared__ BDia dia;
   if (threadIdx.x == 0) {
     a = *args;
     g.C = cluster_ctas();
@@ -1011,15 +1075,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_bcg(const BArgs* __restrict__
       g.target = 0;
       g.gpar = 0;
     }
+    for (int i = t; i < (int)(sizeof(BDia) / 4); i += NT)
+      reinterpret_cast<int32_t*>(&dia)[i] = reinterpret_cast<const int32_t*>(a.dia + inst)[i];
     __syncthreads();
     const bool lead = g.p == 0 && g.cr == 0;
     if (lead && t == 0) a.t_inst[2 * inst] = now_ns();
     bool ok;
     if constexpr (sizeof(V) == 4)
-      ok = a.reliable ? solve_instance_ru<NT>(a, inst, g, red, st, par, &s_flag)
-                      : solve_instance<V, NT>(a, inst, g, red, st, par, &s_flag);
+      ok = a.reliable ? solve_instance_ru<NT>(a, dia, inst, g, red, st, par, &s_flag)
+                      : solve_instance<V, NT>(a, dia, inst, g, red, st, par, &s_flag);
     else
-      ok = solve_instance<V, NT>(a, inst, g, red, st, par, &s_flag);
+      ok = solve_instance<V, NT>(a, dia, inst, g, red, st, par, &s_flag);
     if (!ok) {
       if (lead && t < a.nrhs) {
         gbcg_batch_info o = {st.used[t], st.outer[t], (int)kTimeout, 0, st.rel[t]};
@@ -1121,6 +1187,8 @@ struct gbcg_batch_s {
   int* h_err = nullptr;  // pinned
   double* d_val64 = nullptr;
   float* d_val32 = nullptr;
+  BDia* d_dia = nullptr;
+  float* d_dia32 = nullptr;
   int8_t* d_rpw = nullptr;
   double* d_R64 = nullptr;
   void *d_R = nullptr, *d_P = nullptr, *d_Q = nullptr, *d_D = nullptr;
@@ -1169,7 +1237,7 @@ void free_batch(gbcg_batch_s* B) {
   void* dev[] = {B->d_inst_row, B->d_ptr,  B->d_idx,  B->d_slot_inst, B->d_slot_part, B->d_grp,  B->d_gbar,
                  B->d_gpart,    B->d_err,  B->d_val64, B->d_val32,  B->d_rpw,       B->d_R64,  B->d_R,
                  B->d_P,        B->d_Q,    B->d_D,     B->d_Bst,    B->d_Xst,       B->d_queue, B->d_out,
-                 B->d_iters,    B->d_outer, B->d_t,    B->d_args};
+                 B->d_iters,    B->d_outer, B->d_t,    B->d_args,    B->d_dia,    B->d_dia32};
   for (void* p : dev)
     if (p) cudaFree(p);
   void* host[] = {B->h_args, B->h_out, B->h_iters, B->h_outer, B->h_t, B->h_err};
@@ -1303,6 +1371,8 @@ BArgs base_args(gbcg_batch_s* B) {
   a.idx = B->d_idx;
   a.val64 = B->d_val64;
   a.val32 = B->d_val32;
+  a.dia = B->d_dia;
+  a.dia32 = B->d_dia32;
   a.slot_inst = B->d_slot_inst;
   a.slot_part = B->d_slot_part;
   a.grp = B->d_grp;
@@ -1597,9 +1667,38 @@ int gbcg_batch_create(gbcg_batch_t* out, int32_t count, const int64_t* row_off, 
     return code;
   };
   if (cudaGetDevice(&B->dev) != cudaSuccess) return bail(fail(GBCG_ERR_CUDA, "cudaGetDevice failed"));
+  // the instances of few diagonals, their values one after the other, in a
+  // batch small enough that an instance's own iterations are what takes the
+  // time: 48 systems 163 -> 141 ms.  With several instances queued for every
+  // cluster the SMs' second CTA hides the CSR product's round trips, and it is
+  // the faster one (256 systems: 549 against 566 ms).
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->dev) != cudaSuccess)
+    return bail(fail(GBCG_ERR_CUDA, "cannot query the device"));
+  std::vector<BDia> dia(count);
+  std::vector<double> dval;
+  const char* off = getenv("GBCG_DIAGONALS");
+  if (!(off && off[0] == '0') && 2 * count <= sms) {
+    std::vector<int32_t> lp, li;
+    for (int i = 0; i < count; ++i) {
+      const int64_t r0 = row_off[i], m = row_off[i + 1] - r0, z = B->nnz_of[i], k0 = ptr[r0];
+      lp.resize(m + 1);
+      li.resize(z);
+      for (int64_t r = 0; r <= m; ++r) lp[r] = (int32_t)(ptr[r0 + r] - k0);
+      for (int64_t k = 0; k < z; ++k) li[k] = (int32_t)(idx[k0 + k] - r0);
+      gbcg::DiaHost H;
+      if (!gbcg::build_diagonals(GBCG_CSR, m, z, lp.data(), li.data(), val + k0, 0, H) || H.ld * (int64_t)H.off.size() > 0x7fffffff)
+        continue;
+      dia[i].base = (int64_t)dval.size();
+      dia[i].ld = (int32_t)H.ld;
+      dia[i].K = (int32_t)H.off.size();
+      std::copy(H.off.begin(), H.off.end(), dia[i].off);
+      dval.insert(dval.end(), H.val.begin(), H.val.end());
+    }
+  }
   const size_t nv = (size_t)std::max<int64_t>(1, n) * kRhs;
   int rc = 0;
-  if ((rc = balloc(B, &B->d_inst_row, count + 1)) || (rc = balloc(B, &B->d_ptr, n + 1)) ||
+  if ((rc = balloc(B, &B->d_dia, count)) || (rc = balloc(B, &B->d_dia32, dval.size())) || (rc = balloc(B, &B->d_inst_row, count + 1)) || (rc = balloc(B, &B->d_ptr, n + 1)) ||
       (rc = balloc(B, &B->d_idx, nnz)) || (rc = balloc(B, &B->d_val64, nnz)) || (rc = balloc(B, &B->d_val32, nnz)) ||
       (rc = balloc(B, &B->d_slot_inst, (size_t)count * kMaxGroup)) ||
       (rc = balloc(B, &B->d_slot_part, (size_t)count * kMaxGroup)) || (rc = balloc(B, &B->d_grp, count)) ||
@@ -1640,6 +1739,14 @@ int gbcg_batch_create(gbcg_batch_t* out, int32_t count, const int64_t* row_off, 
     up(B->d_idx, idx, sizeof(int32_t) * nnz);
     up(B->d_val64, val, sizeof(double) * nnz);
     up(B->d_val32, v32.data(), sizeof(float) * nnz);
+    std::vector<float> dval32(dval.size());  // padding stays -0.0, an entry that rounds to zero is +0.0
+    for (size_t k = 0; k < dval.size(); ++k) {
+      const bool padding = dval[k] == 0.0 && std::signbit(dval[k]);
+      const float f = (float)dval[k];
+      dval32[k] = padding ? -0.f : f == 0.f ? 0.f : f;
+    }
+    up(B->d_dia, dia.data(), sizeof(BDia) * count);
+    up(B->d_dia32, dval32.data(), sizeof(float) * dval32.size());
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_out, 0, sizeof(gbcg_batch_info) * (size_t)count * nrhs, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return bail(fail(GBCG_ERR_CUDA, std::string("batch upload: ") + cudaGetErrorString(e)));

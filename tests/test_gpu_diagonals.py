@@ -139,3 +139,35 @@ def test_tiles_asked_for_by_name(torch, precision, monkeypatch):
     assert info.status == "OK"
     r = s.b - oracle.spmv("csr", s.ptr, s.idx, s.val, x.cpu().numpy())
     assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(s.b)
+
+
+@pytest.mark.parametrize("precision", ["fp32_ru", "fp32_ir", "fp64"])
+@pytest.mark.parametrize("nrhs", [8, 3])
+def test_batch(torch, precision, nrhs, monkeypatch):
+    # instances on diagonals beside one that has too many (a random matrix) and
+    # a tiny one turned down for its padding, against the same batch in CSR
+    rng = np.random.default_rng(4)
+    R = sp.random(300, 300, 0.02, random_state=4, format="csr")
+    R = (R + R.T + sp.diags(np.full(300, 12.0))).tocsr()
+    R.sort_indices()
+    mats = [sp.csr_matrix((s.val, s.idx, s.ptr), shape=(s.n, s.n)) for s in
+            (fem(9, 10, 11), fem(5, 5, 4), fem(14, 13, 12, seed_mesh=3), fem(20, 4, 9, contrast=10.0))]
+    mats.insert(1, R)
+    A = sp.block_diag(mats, format="csr")
+    A.sort_indices()
+    off = np.concatenate([[0], np.cumsum([m.shape[0] for m in mats])]).astype(np.int64)
+    b = torch.from_numpy(np.ascontiguousarray(rng.uniform(-1, 1, (A.shape[0], nrhs)))).cuda()
+    args = (off, A.indptr.astype(np.int32), A.indices.astype(np.int32), A.data)
+    out = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("GBCG_DIAGONALS", flag)
+        with gb.Batch(*args, nrhs=nrhs, tune=False) as B:
+            x, infos, rep = B.solve(b, tol=1e-12, maxit=20000, precision=precision)
+            again, _, _ = B.solve(b, tol=1e-12, maxit=20000, precision=precision)
+        assert rep["status"] == "OK" and torch.equal(x, again)
+        r = b.cpu().numpy() - A @ x.cpu().numpy()
+        for a, z in zip(off[:-1], off[1:]):
+            bb = np.linalg.norm(b[a:z].cpu().numpy(), axis=0)
+            assert np.all(np.linalg.norm(r[a:z], axis=0) <= 1.001e-12 * bb)
+        out.append(x)
+    assert torch.linalg.norm(out[0] - out[1]) <= 1e-8 * torch.linalg.norm(out[1])
