@@ -21,7 +21,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgbcg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = [os.path.join(CSRC, f) for f in ("gbcg.cu", "static_solve.cu", "batch.cu", "grad.cu", "ablation.cu", "layout.cpp",
-                                              "kernels.cuh", "diagonals.cuh", "dia_solve.cuh", "fp64.cuh", "layout.h")]
+                                              "kernels.cuh", "diagonals.cuh", "chip_solve.cuh", "fp64.cuh", "layout.h")]
 HEADERS = [os.path.join(INCLUDE, "gbcg.h")]
 
 

@@ -1,5 +1,6 @@
-// dia_solve.cuh -- the persistent conjugate-gradient solvers of the diagonal
-// layout whose vectors stay on the chip.
+// chip_solve.cuh -- the persistent conjugate-gradient solvers whose vectors
+// stay on the chip, on the diagonal layout and, for short ranges of rows per
+// CTA, on the row-gather layout.
 //
 // One CTA per SM owns a contiguous range of rows and keeps those rows of x,
 // r, p and q = A p in shared memory for the whole solve; thread t owns rows
@@ -234,8 +235,12 @@ enum { kSolveFull = 0, kSolveInner = 1, kSolveRu = 2 };
 
 template <typename V>
 struct ChipArgs {
-  DiaDev<V> D;
+  DiaDev<V> D;         // kDia, kDiaSym
   DiaDev<double> D64;  // kSolveRu
+  OpDev<V> A;          // kGather
+  OpDev<double> A64;   // kSolveRu
+  const int32_t* cta_slice;
+  const int32_t* cta_long;
   V* x;                // kSolveFull: the caller's x; kSolveInner: the correction (out)
   const V* b;
   V* p;                // p in global memory
@@ -244,31 +249,88 @@ struct ChipArgs {
   double* xh;          // kSolveRu: x within a halo, for the update's product
   ChipSync* sync;
   CgState* st;
-  int64_t nslices;
+  int32_t n;
   double tol, delta;
   int32_t maxit, max_restarts;
   int32_t rows;        // greatest number of rows of a CTA
   long long timeout_ns;
 };
 
-// First row of CTA c: whole slices, as many for each CTA as the counts allow.
-__host__ __device__ inline int64_t chip_row(int64_t nslices, int c, int G) { return nslices * c / G * 32; }
-// Shared memory of a CTA: four vectors of its rows, the sums' buffers.
+// Shared memory of a CTA: four vectors of its rows, the sums' buffers, the
+// offsets of its slices (row gather).
 template <typename V>
 size_t chip_smem(int64_t rows, int threads) {
-  return 4 * (size_t)rows * sizeof(V) + ((size_t)threads + kMaxSums + 1) * sizeof(double);
+  return 4 * (size_t)rows * sizeof(V) + ((size_t)threads + kMaxSums + 1 + rows / 32 + 1) * sizeof(double);
 }
+
+// f(row, (A x)_row) over the slices of rows [r0, r1) (their offsets in shared
+// memory) and the long rows [l0, l1) of the row-gather layout, straight from
+// global memory: eight entries' columns and values, then their gathers, are
+// in flight together.  The bulk-copy pipeline of spmv_rows keeps more bytes in
+// flight over long ranges; with one or two slices per warp its stage wait only
+// adds to the chain.
+template <typename V, class F>
+__device__ __forceinline__ void chip_gather(const OpDev<V>& A, const int64_t* off, int r0, int r1, int l0, int l1,
+                                            const V* x, F&& f) {
+  constexpr int C = 8;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int s = warp; r0 + 32 * s < r1; s += nw) {
+    const int64_t beg = off[s];
+    const int L = (int)((off[s + 1] - beg) >> 5), row = r0 + 32 * s + lane;
+    const V* __restrict__ val = A.val + beg + lane;
+    V acc = V(0);
+    auto terms = [&](auto* __restrict__ col, const V* xb) {
+      for (int k0 = 0; k0 < L; k0 += C) {
+        V v[C], xv[C];
+        int c[C];
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+          const int k = min(k0 + j, L - 1);
+          c[j] = __ldg(col + 32 * k);
+          v[j] = __ldg(val + 32 * k);
+        }
+#pragma unroll
+        for (int j = 0; j < C; ++j) xv[j] = xb[c[j]];
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+          if (k0 + j < L) acc = dia_fma(v[j], xv[j], acc);
+      }
+    };
+    // 16-bit offsets count from the row (lanes past the last row read x[0])
+    if (A.col16) terms(A.col16 + beg + lane, x + (row < r1 ? row : 0));
+    else terms(A.col + beg + lane, x);
+    if (row < r1 && !((A.long_mask[(r0 >> 5) + s] >> lane) & 1u)) f(row, acc);
+  }
+  for (int li = l0 + warp; li < l1; li += nw) {
+    const V v = long_row<V, false>(A, li, lane, x);
+    if (lane == 0) f((int)A.long_row[li], v);
+  }
+}
+
+// The matrix as a CTA sees it.
+template <typename V, int FMT>
+struct ChipMat {
+  const DiaTab<V>& tab;
+  const OpDev<V>& A;
+  const int64_t* off;
+  int r0, r1, l0, l1;
+  template <bool HALO, int C, int R, class F>
+  __device__ __forceinline__ void rows(const V* x, F&& f) const {
+    if constexpr (is_dia(FMT)) dia_rows<FMT == kDiaSym, HALO, C, R>(tab, r0, r1, x, f);
+    else chip_gather(A, off, r0, r1, l0, l1, x, f);
+  }
+};
 
 // kSolveRu: float(b - A x) of the CTA's rows in double precision, into sr; the
 // thread's sums of the residual's square (before and after rounding) and b's.
 // A function of its own: a dozen calls per solve, and its registers would
 // crowd the iterations'.
-template <typename V, bool SYM>
-__device__ __noinline__ void chip_residual64(const DiaTab<double>& t, int r0, int r1, const double* b, const double* x,
-                                             V* sr, double* sums) {
+template <typename V, int FMT>
+__device__ __noinline__ void chip_residual64(const ChipMat<double, FMT>& M, const double* b, const double* x, V* sr,
+                                             double* sums) {
   double tt = 0.0, bb = 0.0;
   V rr = V(0);
-  dia_rows<SYM, true, 8, 1>(t, r0, r1, x, [&](int i, double q) {
+  M.template rows<true, 8, 1>(x, [&](int i, double q) {
     const double bi = b[i], ti = bi - q;
     const V tf = (V)ti;
     sr[i] = tf;
@@ -281,8 +343,8 @@ __device__ __noinline__ void chip_residual64(const DiaTab<double>& t, int r0, in
   sums[2] = bb;
 }
 
-template <typename V, bool SYM, int KIND, int R>
-__global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_constant__ ChipArgs<V> a) {
+template <typename V, int FMT, int KIND, int R>
+__global__ void __launch_bounds__(chip_threads(R), 1) k_cg_chip(const __grid_constant__ ChipArgs<V> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ DiaTab<V> tab;
   __shared__ DiaTab<double> tab64;
@@ -292,9 +354,8 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
   } sc;  // the step's scalars, formed by thread 0 as a grid sum ends
   __shared__ int sok;
   __shared__ unsigned long long sbase[4];
-  const int c = blockIdx.x, G = gridDim.x, t = threadIdx.x, T = blockDim.x;
-  const int r0 = (int)chip_row(a.nslices, c, G), rend = (int)chip_row(a.nslices, c + 1, G);
-  const int r1 = rend < (int)a.D.n ? rend : (int)a.D.n;
+  const int c = blockIdx.x, t = threadIdx.x, T = blockDim.x;
+  const int r0 = a.cta_slice[c] * 32, r1 = min(a.cta_slice[c + 1] * 32, a.n);
   constexpr int C = R == 1 ? 8 : 16 / (R * (int)sizeof(V));  // diagonals whose loads are in flight together
   GridSum g;
   g.sync = a.sync;
@@ -306,12 +367,19 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
   g.base = sbase;
   if (t < 4) sbase[t] = 0;
   g.timeout_ns = a.timeout_ns;
-  V* sx = reinterpret_cast<V*>(g.out + kMaxSums + 1) - r0;  // indexed by row
+  int64_t* off = reinterpret_cast<int64_t*>(g.out + kMaxSums + 1);
+  V* sx = reinterpret_cast<V*>(off + a.rows / 32 + 1) - r0;  // indexed by row
   V* sr = sx + a.rows;
   V* sq = sr + a.rows;
   V* sp = sq + a.rows;
-  dia_tab_init(tab, a.D);
-  if constexpr (KIND == kSolveRu) dia_tab_init(tab64, a.D64);
+  const int l0 = FMT == kGather ? a.cta_long[c] : 0, l1 = FMT == kGather ? a.cta_long[c + 1] : 0;
+  if constexpr (is_dia(FMT)) {
+    dia_tab_init(tab, a.D);
+    if constexpr (KIND == kSolveRu) dia_tab_init(tab64, a.D64);
+  } else {
+    for (int s = t; s <= (r1 - r0 + 31) / 32; s += T) off[s] = a.A.sl_ptr[r0 / 32 + s];
+  }
+  const ChipMat<V, FMT> M{tab, a.A, off, r0, r1, l0, l1};
   __syncthreads();
   int status = kOk, k = 0, restarts = 0;
   double rr = 0.0, nb = 0.0, rel = 0.0, rmax = 0.0, beta = 0.0, pq = 0.0;
@@ -321,7 +389,7 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
   // kSolveFull: r = b - A x from the x in global memory; returns r'r
   auto residual = [&](double& tt, double& bb) {
     V ptt = V(0), pbb = V(0);
-    dia_rows<SYM, false, C, R>(tab, r0, r1, (const V*)a.x, [&](int i, V q) {
+    M.template rows<false, C, R>((const V*)a.x, [&](int i, V q) {
       const V bi = a.b[i];
       const V ri = bi - q;
       sr[i] = ri;
@@ -342,7 +410,8 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
     }
     if (!chip_barrier(g)) return false;  // x of every CTA
     double v[3];
-    chip_residual64<V, SYM>(tab64, r0, r1, a.b64, a.xh, sr, v);
+    const ChipMat<double, FMT> M64{tab64, a.A64, off, r0, r1, l0, l1};
+    chip_residual64<V, FMT>(M64, a.b64, a.xh, sr, v);
     if (!chip_sum<3>(g, v)) return false;
     const double tt = g.out[0];
     rr = g.out[1];
@@ -422,7 +491,7 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_dia_chip(const __grid_co
       double v[1];
       {
         V ppq = V(0);
-        dia_rows<SYM, true, C, R>(tab, r0, r1, (const V*)a.p, [&](int i, V q) {
+        M.template rows<true, C, R>((const V*)a.p, [&](int i, V q) {
           sq[i] = q;
           ppq = dia_fma(sp[i], q, ppq);
         });

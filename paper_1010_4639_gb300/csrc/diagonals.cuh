@@ -119,14 +119,15 @@ __device__ __forceinline__ void dia_tab_init(DiaTab<V>& t, const DiaDev<V>& A) {
 // Rows i, i + 32, ... (R of them): acc[r] gains the terms of half a row, in
 // increasing column order -- MIRROR: columns i - off[k], k = K - 1 .. 1, whose
 // values rows i - off[k] hold; else columns i + off[k], k = 0 .. K - 1.  The
-// loads of C diagonals are issued before the first is used.  CLAMP (segments
+// loads of C diagonals are issued before the first is used.  DESC: k from K - 1
+// down.  CLAMP (segments
 // at the ends of the matrix): rows past `last` are taken as `last`, columns
 // outside the matrix as its first or last one; the value there is padding (a
 // diagonal is stored with max(off) padding after its n values, where the
 // mirrored index of the rows below off[k] leads).  A branch per diagonal
 // around the clamps, or reading the CTA's own columns from shared memory, were
 // both slower (25 000 -> 31 000 cycles per product at 128^3).
-template <bool MIRROR, bool NC, bool CLAMP, int C, int R, typename V, class E>
+template <bool MIRROR, bool NC, bool CLAMP, bool DESC, int C, int R, typename V, class E>
 __device__ __forceinline__ void dia_half(const E& table, int K, const V* val, int n, int last, int i0, const V* x,
                                          V (&acc)[R]) {
   const E entry = table.fresh();
@@ -137,7 +138,7 @@ __device__ __forceinline__ void dia_half(const E& table, int K, const V* val, in
     for (int j = 0; j < C; ++j) {
       // past the last diagonal: the last one again, unused (no branches around the loads)
       const int m = min(kb + j, cnt - 1);
-      const int2 d = entry(MIRROR ? K - 1 - m : m);
+      const int2 d = entry(MIRROR || DESC ? K - 1 - m : m);
       if constexpr (!CLAMP) {
         const int c = MIRROR ? i0 - d.y : i0 + d.y;
         const V* pv = val + ((uint32_t)d.x + (uint32_t)(MIRROR ? c : i0));
@@ -183,8 +184,8 @@ __device__ __forceinline__ V dia_row_exact(const E& table, int K, const V* val, 
     }
   if constexpr (!dia_apart<SYM, V>()) acc = low;
 #pragma unroll 1
-  for (int k = 0; k < K; ++k) {
-    const int2 d = entry(k);
+  for (int m = 0; m < K; ++m) {
+    const int2 d = entry(dia_apart<SYM, V>() ? K - 1 - m : m);
     const int c = i + d.y;
     if (c < 0 || c >= n) continue;
     const V v = __ldg(val + ((uint32_t)d.x + (uint32_t)i));
@@ -205,20 +206,21 @@ __device__ __forceinline__ void dia_segment(const E& entry, int K, int lo, int h
   const int i0 = base + (threadIdx.x & 31);
 #pragma unroll
   for (int r = 0; r < R; ++r) acc[r] = V(0);
-  // single-precision symmetric rows sum the columns below the diagonal apart,
-  // as the tiles do: shorter sums round less (5.6e-8 against 8.1e-8, relative,
-  // on a finite-element matrix); double precision goes on with the same sum,
-  // as full storage does
+  // single-precision symmetric rows sum the columns below and above the
+  // diagonal apart and take the diagonal, the largest term, last, as the tiles
+  // do: shorter and smaller sums round less (one sum: 8.1e-8 on a
+  // finite-element matrix, the tiles 5.5e-8); double precision goes on with one sum, as full
+  // storage does
   constexpr bool kApart = dia_apart<SYM, V>();
   V low[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) low[r] = V(0);
   if (HALO || (base + lo >= 0 && base + 32 * R - 1 + hi < n && base + 32 * R - 1 <= last)) {
-    if constexpr (SYM) dia_half<true, NC, false, C, R>(entry, K, val, n, last, i0, x, kApart ? low : acc);
-    dia_half<false, NC, false, C, R>(entry, K, val, n, last, i0, x, acc);
+    if constexpr (SYM) dia_half<true, NC, false, false, C, R>(entry, K, val, n, last, i0, x, kApart ? low : acc);
+    dia_half<false, NC, false, kApart, C, R>(entry, K, val, n, last, i0, x, acc);
   } else {
-    if constexpr (SYM) dia_half<true, NC, true, C, R>(entry, K, val, n, last, i0, x, kApart ? low : acc);
-    dia_half<false, NC, true, C, R>(entry, K, val, n, last, i0, x, acc);
+    if constexpr (SYM) dia_half<true, NC, true, false, C, R>(entry, K, val, n, last, i0, x, kApart ? low : acc);
+    dia_half<false, NC, true, kApart, C, R>(entry, K, val, n, last, i0, x, acc);
   }
   if constexpr (kApart)
 #pragma unroll

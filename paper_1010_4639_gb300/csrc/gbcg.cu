@@ -17,7 +17,7 @@
 #include <vector>
 
 #include "../../include/gbcg.h"
-#include "dia_solve.cuh"
+#include "chip_solve.cuh"
 #include "kernels.cuh"
 #include "layout.h"
 
@@ -258,7 +258,7 @@ struct gbcg_matrix_s {
   ChipSync* sync = nullptr;
   GridBar* bar = nullptr;   // &sync->bar
   CgState* st = nullptr;
-  int64_t chip_rows = 0;    // diagonal layout: greatest number of rows of a CTA
+  int64_t chip_rows = 0;    // greatest number of rows of a CTA, in whole slices
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // brackets of the persistent launches
   // pinned host mirrors
   CgState* st_h = nullptr;
@@ -485,23 +485,34 @@ cudaError_t launch_ru(const RuArgs& args, int grid, cudaStream_t s) {
 // limit less their static variables.
 constexpr size_t kChipSmem = 225 * 1024;
 
-// Whether a CTA's rows of the four vectors fit on the chip (dia_solve.cuh).
+// Rows per CTA up to which the row-gather layout's solves stay on the chip (us
+// per reliable-update iteration, pipeline -> chip, unstructured numbering:
+// 170 rows 11.7 -> 7.3, 560 rows 13.5 -> 9.3, 1 570 rows 17.5 -> 12.7, 3 120
+// rows 23.8 -> 18.2; not measured beyond).
+constexpr int64_t kChipGatherRows = 3200;
+
+// Whether a CTA's rows of the four vectors fit on the chip (chip_solve.cuh).
 template <typename V>
 bool on_chip(const gbcg_matrix_s* M) {
-  return is_dia(M->mode) && M->grid <= kChipCtas && chip_smem<V>(M->chip_rows, kChipThreads) <= kChipSmem;
+  const bool layout = is_dia(M->mode) || (M->mode == kGather && M->chip_rows <= kChipGatherRows);
+  return layout && M->grid <= kChipCtas && chip_smem<V>(M->chip_rows, kChipThreads) <= kChipSmem;
 }
 
-template <typename V, bool SYM, int KIND, int R>
+template <typename V, int FMT, int KIND, int R>
 cudaError_t launch_chip(const gbcg_matrix_s* M, ChipArgs<V> a, cudaStream_t s) {
   a.D = M->dia<V>();
   a.D64 = M->dia<double>();
+  a.A = M->op<V>();
+  a.A64 = M->op<double>();
+  a.cta_slice = M->cta_slice;
+  a.cta_long = M->cta_long;
   a.sync = M->sync;
   a.st = M->st;
-  a.nslices = M->nslices;
+  a.n = (int32_t)M->n;
   a.rows = (int32_t)M->chip_rows;
   const int threads = (int)std::min<int64_t>(chip_threads(R), M->chip_rows);
   const size_t smem = chip_smem<V>(M->chip_rows, threads);
-  const void* kernel = (const void*)k_dia_chip<V, SYM, KIND, R>;
+  const void* kernel = (const void*)k_cg_chip<V, FMT, KIND, R>;
   cudaError_t e = cudaMemsetAsync(M->sync, 0, sizeof(ChipSync), s);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChipSmem);
   if (e != cudaSuccess) return e;
@@ -510,15 +521,15 @@ cudaError_t launch_chip(const gbcg_matrix_s* M, ChipArgs<V> a, cudaStream_t s) {
 }
 template <typename V, int KIND>
 cudaError_t launch_chip_fmt(const gbcg_matrix_s* M, const ChipArgs<V>& a, cudaStream_t s) {
+  if (M->mode == kGather) return launch_chip<V, kGather, KIND, 1>(M, a, s);
   // two rows per thread and product step once 512 threads would take more than
   // four rounds (1024 threads of 64 registers: 36.1 against 38.1 us per FP64
   // iteration, 17.7 against 19.3 single precision, at 5 500 rows per CTA; one
   // row per step and 128 registers for short ranges, where the round trip
   // counts: 8.5 against 10.5 us at 170 rows)
-  constexpr int R = 2;
   if (M->chip_rows > 2048)
-    return M->mode == kDiaSym ? launch_chip<V, true, KIND, R>(M, a, s) : launch_chip<V, false, KIND, R>(M, a, s);
-  return M->mode == kDiaSym ? launch_chip<V, true, KIND, 1>(M, a, s) : launch_chip<V, false, KIND, 1>(M, a, s);
+    return M->mode == kDiaSym ? launch_chip<V, kDiaSym, KIND, 2>(M, a, s) : launch_chip<V, kDia, KIND, 2>(M, a, s);
+  return M->mode == kDiaSym ? launch_chip<V, kDiaSym, KIND, 1>(M, a, s) : launch_chip<V, kDia, KIND, 1>(M, a, s);
 }
 
 // Product y = A x (MODE 0), or r = b - A x into y with per-CTA partial sums
@@ -968,8 +979,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
     TRY(upload(&M->dia32, dia_to_f32(Dh.val), s, B));
     // every row costs the same: equal ranges of whole slices
     cs.resize(M->grid + 1);
-    for (int c = 0; c <= M->grid; ++c) cs[c] = (int32_t)(chip_row(M->nslices, c, M->grid) / 32);
-    for (int c = 0; c < M->grid; ++c) M->chip_rows = std::max<int64_t>(M->chip_rows, 32 * (int64_t)(cs[c + 1] - cs[c]));
+    for (int c = 0; c <= M->grid; ++c) cs[c] = (int32_t)(M->nslices * c / M->grid);
   } else {
     TRY(upload(&M->sl_ptr, L.A.sl_ptr, s, B));
     TRY(upload(&M->col, L.A.col, s, B));
@@ -999,6 +1009,8 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
     TRY(upload(&M->diag64, L.diag, s, B));
     TRY(upload(&M->diag32, to_f32(L.diag), s, B));
   }
+  M->chip_rows = 32;
+  for (int c = 0; c < M->grid; ++c) M->chip_rows = std::max<int64_t>(M->chip_rows, 32 * (int64_t)(cs[c + 1] - cs[c]));
   TRY(upload(&M->cta_slice, cs, s, B));
   TRY(upload(&M->cta_long, cl, s, B));
   // workspace
