@@ -1075,8 +1075,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_bcg(const BArgs* __restrict__
       g.target = 0;
       g.gpar = 0;
     }
-    for (int i = t; i < (int)(sizeof(BDia) / 4); i += NT)
-      reinterpret_cast<int32_t*>(&dia)[i] = reinterpret_cast<const int32_t*>(a.dia + inst)[i];
+    // A probe of one rows-per-warp choice takes the CSR product of every
+    // instance: the choice serves the double-precision solve and the
+    // residuals, which have no diagonals.
+    if (a.force_rpw > 0) {
+      if (t == 0) dia.K = 0;
+    } else {
+      for (int i = t; i < (int)(sizeof(BDia) / 4); i += NT)
+        reinterpret_cast<int32_t*>(&dia)[i] = reinterpret_cast<const int32_t*>(a.dia + inst)[i];
+    }
     __syncthreads();
     const bool lead = g.p == 0 && g.cr == 0;
     if (lead && t == 0) a.t_inst[2 * inst] = now_ns();
@@ -1398,8 +1405,9 @@ BArgs base_args(gbcg_batch_s* B) {
 }
 
 // One probe launch (not captured): every instance runs `iters` inner
-// iterations of one refinement pass with rows-per-warp `rpw` (0: the
-// per-instance table).  Returns the launch time and fills h_t.
+// iterations of one refinement pass with rows-per-warp `rpw` on the CSR
+// product (0: the per-instance table, and the diagonals where they serve).
+// Returns the launch time and fills h_t.
 int probe(gbcg_batch_s* B, bool f32, int threads, int cluster, int clusters, int rpw, int iters, const double* Bp,
           double* Xp, cudaStream_t s, float* ms) {
   if (int rc = single_schedule(B, s)) return rc;
