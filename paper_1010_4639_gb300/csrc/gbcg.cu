@@ -81,6 +81,13 @@ std::vector<float> dia_to_f32(const std::vector<double>& v) {
 // Tile caps of each precision's layout (the kernels' TileCaps).
 constexpr int kTileSlices32 = kTileWarps * TileCaps<float>::kRpt, kTileSlices64 = kTileWarps * TileCaps<double>::kRpt;
 
+// Windows per tile (layout.h, sym_windows) up to which symmetric storage
+// is computed by tiles.  Twice what a tile's descriptor holds; a mesh numbered
+// line by line has 3 or 4, one renumbered at random within 2048 unknowns some
+// 100, where a reliable-update iteration of 85 000 rows took 435 us in tiles
+// and takes 9 with the full operator's row gather.
+constexpr double kTileWindows = 2 * kDescWin;
+
 int env_int(const char* name, int dflt) {
   const char* s = getenv(name);
   return (s && *s) ? atoi(s) : dflt;
@@ -212,7 +219,7 @@ struct gbcg_matrix_s {
   double* u_stage = nullptr;
   int64_t nslices = 0, nlong = 0, bytes = 0;
   int sym = 0;
-  int mode = kGather;       // kGather or kDia (CSR/CSC), kPlan, kTiles or kDiaSym (symmetric)
+  int mode = kGather;       // kGather or kDia; symmetric: also kPlan, kTiles or kDiaSym
   int64_t l2_bytes = 0;     // the device's L2 size
   // tiled symmetric layouts (device): single- and double-precision products
   DevTiles t32, t64;
@@ -899,7 +906,15 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
   const bool sym_named = format == GBCG_SYM_CSR_UPPER && sym_mode && *sym_mode;
   const bool diagonals = !sym_named && env_int("GBCG_DIAGONALS", 1) != 0 &&
                          build_diagonals(format, n, nnz, ptr, idx, val, index_base, Dh);
-  if (!diagonals && (rc = build_layout(format, n, nnz, ptr, idx, val, index_base, L, err)) != 0) return fail(rc, err);
+  // symmetric storage whose neighbours are scattered takes the full operator's
+  // row-gather layout in place of tiles (the caps of the double-precision
+  // tiles are the tighter ones; what fits no tile keeps the transpose plan)
+  const bool sym_full = !diagonals && format == GBCG_SYM_CSR_UPPER && !sym_named &&
+                        sym_windows(n, ptr, idx, index_base) > kTileWindows &&
+                        sym_slices_fit(n, ptr, idx, index_base, TileCaps<double>::kSlot, TileCaps<double>::kEnt) &&
+                        build_sym_full(n, nnz, ptr, idx, val, index_base, L);
+  if (!diagonals && !sym_full && (rc = build_layout(format, n, nnz, ptr, idx, val, index_base, L, err)) != 0)
+    return fail(rc, err);
   // debug mode: full CSR/CSC inputs must be symmetric (CG's premise)
   if (format != GBCG_SYM_CSR_UPPER && env_int("GBCG_CHECK_SYMMETRY", 0) != 0 &&
       (rc = check_symmetry(n, nnz, ptr, idx, val, index_base, err)) != 0)
@@ -937,7 +952,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
     return bail(fail(GBCG_ERR_CUDA, "cannot query the device"));
   M->l2_bytes = l2;
-  M->mode = diagonals ? (M->sym ? kDiaSym : kDia) : !M->sym ? kGather : (sym_mode && !strcmp(sym_mode, "plan")) ? kPlan : kTiles;
+  M->mode = diagonals ? (M->sym ? kDiaSym : kDia) : !M->sym || sym_full ? kGather : (sym_mode && !strcmp(sym_mode, "plan")) ? kPlan : kTiles;
   auto choose_grid = [&]() -> int {
     if (int rc = mode_occupancy(M->mode, per_sm)) return rc;
     if (per_sm < 1) return fail(GBCG_ERR_CUDA, "the persistent solver kernel cannot be resident");
@@ -1005,7 +1020,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
     }
     cl[M->grid] = (int32_t)M->nlong;
   }
-  if (M->sym && !diagonals) {
+  if (M->sym && !diagonals && !sym_full) {
     TRY(upload(&M->diag64, L.diag, s, B));
     TRY(upload(&M->diag32, to_f32(L.diag), s, B));
   }
@@ -1032,7 +1047,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
   TRY(dalloc(&M->q32, nn, B));
   TRY(dalloc(&M->d32, nn, B));
   TRY(dalloc(&M->rhs32, nn, B));
-  if (M->mode != kTiles && M->mode != kDiaSym) {  // the single-reduction CG's vectors
+  if (!M->sym || M->mode == kPlan) {  // the single-reduction CG's vectors
     TRY(dalloc(&M->s64, nn, B));
     TRY(dalloc(&M->z64, nn, B));
     TRY(dalloc(&M->w64a, nn, B));
@@ -1085,7 +1100,7 @@ int check_solve_opts(const gbcg_matrix_s* A, const gbcg_opts* opts) {
     return fail(GBCG_ERR_INVALID,
                 "the single-reduction variant is double precision only: in single precision its recurrences "
                 "drift past any useful inner tolerance");
-  if (opts && opts->variant == GBCG_PIPELINED && (A->mode == kTiles || A->mode == kDiaSym))
+  if (opts && opts->variant == GBCG_PIPELINED && A->sym && A->mode != kPlan)
     return fail(GBCG_ERR_INVALID,
                 "the single-reduction variant runs on row-gather layouts (CSR, CSC, or symmetric storage with "
                 "GBCG_SYM_LAYOUT=plan); the tiled symmetric product needs a barrier of its own");
@@ -1178,13 +1193,13 @@ int gbcg_stats(gbcg_matrix_t A, gbcg_matrix_stats* out) {
   const int64_t n = A->n, m = A->nnz_input;
   // the product's matrix stream: value + column index per entry (2-byte
   // offsets in the row-gather layout when they fit), row pointers, x, y
-  const int64_t ib = A->narrow ? 2 : 4;
+  const int64_t ib = A->narrow && !A->sym ? 2 : 4;
   out->spmv_bytes_fp64 = (8 + ib) * m + 4 * (n + 1) + 16 * n;
   out->spmv_bytes_fp32 = (4 + ib) * m + 4 * (n + 1) + 8 * n;
   out->index_bytes = (int32_t)ib;
   out->format = A->format;
   out->grid_ctas = A->grid;
-  out->layout = A->mode == kDia ? kGather : A->mode == kDiaSym ? kTiles : A->mode;
+  out->layout = !A->sym ? kGather : A->mode == kPlan ? kPlan : kTiles;
   out->tiles = (int32_t)A->t64.ntiles;  // the double-precision layout's (the single-precision one has about half)
   out->ext_slots = A->t64.next;
   return GBCG_OK;
@@ -1210,6 +1225,9 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
     if (diagonals) {
       if (!build_diagonals(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, Dh))
         return fail(GBCG_ERR_INVALID, "rebuilding the value map: diagonals differ from the handle's");
+    } else if (A->sym && A->mode == kGather) {
+      if (!build_sym_full(A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, L))
+        return fail(GBCG_ERR_INVALID, "rebuilding the value map: layout differs from the handle's");
     } else if (int rc = build_layout(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base,
                                      L, err)) {
       return fail(rc, "rebuilding the value map: " + err);
@@ -1243,7 +1261,7 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
         A->u_len_long = (int64_t)L.A.long_val.size();
       }
     }
-    if (A->sym && !diagonals) {
+    if (A->sym && !diagonals && A->mode != kGather) {
       if (int rc = upload(&A->u_map_diag, to_map(L.diag), s, B)) return rc;
       A->u_len_diag = (int64_t)L.diag.size();
     }

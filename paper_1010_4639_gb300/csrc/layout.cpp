@@ -263,6 +263,51 @@ int check_symmetry(int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* id
   return 0;
 }
 
+bool build_sym_full(int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val, int32_t base,
+                    LayoutHost& out) {
+  if (2 * nnz > 0x7fffffffLL) return false;
+  out = LayoutHost();
+  out.format = 1;
+  out.n = n;
+  out.nnz_input = nnz;
+  Rows R;
+  R.rp.assign(n + 1, 0);
+  int64_t zero_diag = 0;
+  for (int64_t r = 0; r < n; ++r)
+    for (int64_t k = (int64_t)ptr[r] - base; k < (int64_t)ptr[r + 1] - base; ++k) {
+      const int64_t c = (int64_t)idx[k] - base;
+      ++R.rp[r + 1];
+      if (c != r) ++R.rp[c + 1];
+      else zero_diag += val[k] == 0.0;
+    }
+  for (int64_t r = 0; r < n; ++r) R.rp[r + 1] += R.rp[r];
+  R.rc.resize(R.rp[n]);
+  R.rv.resize(R.rp[n]);
+  std::vector<int64_t> fill(R.rp.begin(), R.rp.end() - 1);
+  auto put = [&](int64_t r, int64_t c, double v) {
+    R.rc[fill[r]] = (int32_t)c;
+    R.rv[fill[r]++] = v;
+  };
+  // a row's lower entries come from the rows above it, in increasing order;
+  // its own upper entries follow, and its diagonal
+  for (int64_t r = 0; r < n; ++r) {
+    int64_t kd = -1;
+    for (int64_t k = (int64_t)ptr[r] - base; k < (int64_t)ptr[r + 1] - base; ++k) {
+      const int64_t c = (int64_t)idx[k] - base;
+      if (c == r) {
+        kd = k;
+        continue;
+      }
+      put(r, c, val[k]);
+      put(c, r, val[k]);
+    }
+    if (kd >= 0) put(r, r, val[kd]);
+  }
+  out.nnz_full = R.rp[n] - zero_diag;
+  slice_rows(n, R, true, out.A);
+  return true;
+}
+
 int build_layout(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                  const double* val, int32_t base, LayoutHost& out, std::string& err) {
   int rc = validate_input(format, n, nnz, ptr, idx, val, base, err);
@@ -394,6 +439,65 @@ void make_windows(const std::vector<int32_t>& tg, int64_t n, std::vector<Window>
     i = j;
   }
 }
+
+}  // namespace
+
+double sym_windows(int64_t n, const int32_t* ptr, const int32_t* idx, int32_t base) {
+  // a tile's rows: 15 slices, or what a CTA of 152 gets of a small matrix
+  const int64_t slices = ((n + 31) / 32 + 151) / 152, kRows = 32 * std::min<int64_t>(15, std::max<int64_t>(1, slices));
+  std::vector<int32_t> tg;
+  std::vector<Window> wins;
+  int64_t blocks = 0, windows = 0;
+  // a block in every 8, and every block of a small matrix
+  const int64_t step = n > 64 * kRows ? 8 * kRows : kRows;
+  for (int64_t a = 0; a < n; a += step) {
+    const int64_t b = std::min(n, a + kRows);
+    tg.clear();
+    for (int64_t r = a; r < b; ++r)
+      for (int64_t k = (int64_t)ptr[r] - base; k < (int64_t)ptr[r + 1] - base; ++k)
+        if ((int64_t)idx[k] - base >= b) tg.push_back(idx[k] - base);
+    std::sort(tg.begin(), tg.end());
+    tg.erase(std::unique(tg.begin(), tg.end()), tg.end());
+    make_windows(tg, n, wins);
+    windows += (int64_t)wins.size();
+    ++blocks;
+  }
+  return blocks ? (double)windows / (double)blocks : 0.0;
+}
+
+bool sym_slices_fit(int64_t n, const int32_t* ptr, const int32_t* idx, int32_t base, int slot_cap, int ent_cap) {
+  std::vector<int32_t> tg;
+  std::vector<Window> wins;
+  for (int64_t a = 0; a < n; a += 32) {
+    const int64_t b = std::min(n, a + 32);
+    int64_t longest = 0;
+    tg.clear();
+    for (int64_t r = a; r < b; ++r) {
+      int64_t len = 0;
+      for (int64_t k = (int64_t)ptr[r] - base; k < (int64_t)ptr[r + 1] - base; ++k)
+        if ((int64_t)idx[k] - base != r) {
+          tg.push_back(idx[k] - base);
+          ++len;
+        }
+      longest = std::max(longest, len);
+    }
+    std::sort(tg.begin(), tg.end());
+    int64_t hits = 0, run = 0;  // of the column most rows reach
+    for (size_t i = 0; i < tg.size(); ++i) {
+      run = i > 0 && tg[i] == tg[i - 1] ? run + 1 : 1;
+      hits = std::max(hits, run);
+    }
+    tg.erase(std::unique(tg.begin(), tg.end()), tg.end());
+    tg.erase(tg.begin(), std::lower_bound(tg.begin(), tg.end(), (int32_t)b));
+    make_windows(tg, n, wins);
+    int64_t slots = ((b - a) + 3) & ~int64_t(3);
+    for (const Window& w : wins) slots += w.len;
+    if (slots > slot_cap || 32 * std::max(longest, hits) > ent_cap) return false;
+  }
+  return true;
+}
+
+namespace {
 
 // Colours the entries of one tile so that, in every colour (round), each
 // row has at most one entry and each target slot receives at most one:

@@ -173,6 +173,23 @@ int validate_input(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, c
 bool build_diagonals(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                      const double* val, int32_t index_base, DiaHost& out);
 
+// Windows of a tile's rows (480; fewer in a small matrix) of a validated
+// symmetric input, per tile on average: runs of consecutive rows beyond the
+// block that its upper entries reach.  Three or four for a mesh numbered line
+// by line; hundreds when neighbours are scattered, where the tiles' lists of
+// windows and runs cost more than the product.
+double sym_windows(int64_t n, const int32_t* ptr, const int32_t* idx, int32_t index_base);
+
+// Whether every 32-row slice of a validated symmetric input fits a tile of the
+// given caps by itself (build_sym_tiles fails otherwise).
+bool sym_slices_fit(int64_t n, const int32_t* ptr, const int32_t* idx, int32_t index_base, int slot_cap, int ent_cap);
+
+// Builds the row-gather layout of the full operator of a validated symmetric
+// input (each off-diagonal entry stored twice), a row's diagonal entry last.
+// False when it holds more than 2^31 - 1 entries.
+bool build_sym_full(int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
+                    int32_t index_base, LayoutHost& out);
+
 // Validates the input and builds the row-gather (or symmetric) layout.
 // Returns 0 or a gbcg_status error code, with a message in `err`.
 int build_layout(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
