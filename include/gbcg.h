@@ -129,8 +129,9 @@ typedef struct {
   int32_t grid_ctas;          /* CTAs of the persistent CG launch */
   int32_t layout;             /* family: 0 full storage (row gather, or diagonals where the matrix
                                  has few), 1 symmetric transpose plan, 2 default symmetric storage
-                                 (tiles, or diagonals) */
-  int32_t tiles;              /* symmetric tiles: number of tiles (0 on diagonals) */
+                                 (tiles, diagonals, or the full operator's rows where the numbering
+                                 scatters the neighbours) */
+  int32_t tiles;              /* symmetric tiles: number of tiles (0 in the other layouts) */
   int32_t index_bytes;        /* bytes per column index in the product's stream: 2 when the
                                  row-gather layout stores 16-bit offsets from the row (every
                                  offset fits; natural-order finite-element matrices up to
@@ -164,7 +165,8 @@ typedef struct {
  * The library deep-copies the arrays into its own device layout (values by
  * diagonal when the matrix has at most 32 diagonals that are at least two
  * thirds full, as a mesh numbered line by line gives; else a sliced row-gather
- * layout or symmetric tiles; a single-precision copy of the values, the solve
+ * layout, for symmetric storage tiles or, where the numbering scatters the
+ * neighbours, the full operator's row-gather layout; a single-precision copy of the values, the solve
  * workspace); the caller may free its arrays when the call returns.  The
  * environment variables GBCG_DIAGONALS=0 and GBCG_SYM_LAYOUT=tiles|plan keep
  * the other layouts.

@@ -7,17 +7,22 @@
 // values and column indices into shared memory with a bulk asynchronous copy
 // (cp.async.bulk, completion on an mbarrier, L2 evict-first policy) while it
 // computes the current one, so the number of bytes in flight does not depend
-// on how many warps are resident.  The symmetric format is computed by
-// CTA-cooperative tiles (a producer warp streams tile stages; the entries of
-// a tile come in conflict-free rounds, so the transpose half U' x is a
-// shared-memory scatter without atomics, one barrier per round, and sums
-// leaving a tile are added after a grid barrier), or, as a fallback, as a
-// second row gather through a transpose plan that reads U's values in place.  The paper used a separate scatter kernel with atomics;
+// on how many warps are resident.  A matrix of few diagonals is computed by
+// diagonals, in either storage (diagonals.cuh: no indices, and symmetric
+// storage reads each value once from memory and its mirror from L2).  Other
+// symmetric matrices are computed by CTA-cooperative tiles (a producer warp
+// streams tile stages; the entries of a tile come in conflict-free rounds, so
+// the transpose half U' x is a shared-memory scatter without atomics, one
+// barrier per round, and sums leaving a tile are added after a grid barrier),
+// by the full operator's row gather where the neighbours are scattered, or,
+// as a fallback, as a second row gather through a transpose plan that reads
+// U's values in place.  The paper used a separate scatter kernel with atomics;
 // here every output element is summed in a fixed order, so results are
 // bitwise reproducible.
 //
 // CG iteration (Section III listing): one persistent cooperative launch per
-// solve.  Each CTA owns a contiguous range of slices (and so of rows); per
+// solve.  Where a CTA's rows of the vectors fit its shared memory the solve is
+// chip_solve.cuh's; the kernels here keep them in memory.  Each CTA owns a contiguous range of slices (and so of rows); per
 // iteration it runs
 //   A: q = A p on its rows, partial p'q            -> grid barrier
 //   B: alpha = r'r / p'q; x += alpha p; r -= alpha q; partial r'r -> barrier
@@ -52,7 +57,8 @@ constexpr int kStages = 2;   // stages per warp
 constexpr uint16_t kPlanPad = 0xFFFF;
 constexpr int kMaxStages = 3 + 2;  // mbarriers per warp: a single- (3) and a double-precision (2) pipeline
 
-// Layout modes of the product.
+// Layout modes of the product: row gather, transpose plan, symmetric tiles,
+// diagonals of the full operator, diagonals of the upper half.
 enum { kGather = 0, kPlan = 1, kTiles = 2, kDia = 3, kDiaSym = 4 };
 __host__ __device__ constexpr bool is_dia(int fmt) { return fmt == kDia || fmt == kDiaSym; }
 // Threads per CTA of the persistent kernels in a layout mode.
@@ -1210,7 +1216,7 @@ struct Quad {
 };
 
 // ------------------------------------------------ streamed vector passes ---
-// A vector pass of a tiled solver streams its input vectors through shared
+// A vector pass of a tiled or diagonal solver streams its input vectors through shared
 // memory (the tile stages' space, idle between products): one thread issues
 // bulk copies of 8 KB chunks of the arrays (2048 float or 1024 double rows),
 // kVecBufs chunks ahead, so an SM keeps up to kVecBufs x NA x 8 KB of reads in
