@@ -653,7 +653,7 @@ __device__ bool solve_instance(const BArgs& a, const BDia& dia, int inst, Group&
             if (!quick_finite(s) || !quick_positive(s))
               st.bd[t] = 1;
             else
-              al = quick_div<V>(st.rr[t], s);
+              al = quick_div(st.rr[t], s);
           }
           st.alpha[t] = al;
         }
@@ -698,7 +698,7 @@ __device__ bool solve_instance(const BArgs& a, const BDia& dia, int inst, Group&
               if (st.at_tol[t].below(s, [&] { return sqrt(s) <= st.itol[t] * st.nr0[t]; })) {
                 st.beta[t] = 0.0;
               } else {
-                st.beta[t] = quick_div<V>(s, st.rr[t]);
+                st.beta[t] = quick_div(s, st.rr[t]);
                 st.rr[t] = s;
                 go = st.used[t] < st.maxit;
               }
@@ -951,7 +951,7 @@ __device__ bool solve_instance_ru(const BArgs& a, const BDia& dia, int inst, Gro
               st.status[t] = kNotSpd;
               stop = true;
             } else {
-              al = quick_div<float>(st.rr[t], s);
+              al = quick_div(st.rr[t], s);
             }
           }
           st.alpha[t] = al;
@@ -1015,7 +1015,7 @@ __device__ bool solve_instance_ru(const BArgs& a, const BDia& dia, int inst, Gro
     {
       if (t < kRhs) {
         const bool live = !((st.fin >> t) & 1u);
-        st.beta[t] = live ? quick_div<float>(st.nr[t], st.rr[t]) : 0.0;
+        st.beta[t] = live ? quick_div(st.nr[t], st.rr[t]) : 0.0;
         if (live) st.rr[t] = st.nr[t];
       }
       __syncthreads();

@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_cg_chip(const __grid_con
       }
       if (!chip_sum_fast(g, v[0], pq, [&](const double (&s)[1]) {
             sc.code = !quick_finite(s[0]) ? kNonfinite : !quick_positive(s[0]) ? kNotSpd : kOk;
-            sc.alpha = quick_div<V>(rr, s[0]);
+            sc.alpha = quick_div(rr, s[0]);
           }))
         return;
       pq = g.out[0];
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_cg_chip(const __grid_con
             } else {
               sc.code = at_tol.below(z, [&] { return sqrt(z) / nb <= a.tol; }) ? 1 : 0;
             }
-            sc.beta = quick_div<V>(z, rr);
+            sc.beta = quick_div(z, rr);
           }))
         return;
       ++k;
