@@ -142,53 +142,77 @@ __device__ __forceinline__ bool chip_barrier(GridSum& g) {
   return grid_barrier(&g.sync->bar, g.target, g.timeout_ns, g.ok, g.sums);
 }
 
-// chip_sum of one value per thread whose sum is expected within 2^-13 .. 2^20
+// A CTA's partial sum as a fixed-point number whose unit is 2^-72 of the
+// leading bit of `prev` (ep: prev's sign and exponent): 40 low bits, and a
+// signed high part of 47.  kFixMark as the low part when it does not fit
+// (2^15 of prev and above, infinities, NaN).
+constexpr int kFixUnit = 72;  // unit below prev, in bits
+constexpr int kFixFall = 10;  // a sum may be this many bits below prev
+constexpr unsigned long long kFixMark = 1ull << 48;
+struct FixedParts {
+  long long hi;
+  unsigned long long lo;
+};
+__host__ __device__ __forceinline__ FixedParts fixed_parts(double s, int ep) {
+  const unsigned long long bits = double_bits(s);
+  const int es = (int)(bits >> 52) & 0x7ff, sh = es - ep + kFixUnit - 52;
+  const unsigned long long m = (bits & 0xfffffffffffffull) | (1ull << 52), low40 = (1ull << 40) - 1;
+  FixedParts f = {0, 0};
+  if (sh > 34) {
+    f.lo = kFixMark;
+  } else if (es > 0 && sh > -53) {
+    const unsigned long long w = sh < 0 ? m >> -sh : m;
+    const int up = sh < 0 ? 0 : sh;
+    f.lo = (w << up) & low40;
+    f.hi = (long long)(w >> (40 - up));
+    if ((long long)bits < 0) {
+      f.hi = f.lo ? -f.hi - 1 : -f.hi;
+      f.lo = (0 - f.lo) & low40;
+    }
+  }
+  return f;
+}
+// The sum of such parts as a double; `again`: it was marked, or is less than
+// 2^-10 of prev (or negative), where the parts' truncations would count.
+__host__ __device__ __forceinline__ double fixed_value(FixedParts sum, int ep, bool& again) {
+  const double unit = bits_double((uint64_t)(ep - kFixUnit) << 52);  // powers of two scale exactly
+  const double v = fma((double)sum.hi, unit * 0x1p40, (double)(long long)sum.lo * unit);
+  again = sum.lo >= kFixMark || (int)((long long)double_bits(v) >> 52) < ep - kFixFall;
+  return v;
+}
+
+// chip_sum of one value per thread whose sum is expected within 2^-10 .. 2^14
 // of `prev` (the same sum an iteration earlier), without a memory fence: it
 // orders nothing but the sum itself.  Each CTA adds its partial sum to two
-// 64-bit integers with relaxed atomics, as a fixed-point number of 87 bits
-// whose unit is 2^-67 of prev (a high part and 40 low bits), and each word
-// counts its arrivals in its low 8 bits; a CTA polls the two words until both
-// counts are full and has the sum.  Integer addition makes the sum independent
-// of the order of arrival, and it is exact to 2^-59 of prev or better, closer
-// than a chain of FP64 additions.  This replaces a store of the partial sum,
-// the fence that publishes it, a poll, a load of all partial sums and their
-// additions: 5 100 -> 2 900 cycles per sum with 152 CTAs.  A partial sum out
-// of range marks the low word; a marked or unexpectedly small sum is taken
-// again by chip_sum, by every CTA alike.
+// 64-bit integers with relaxed atomics, as a fixed-point number (fixed_parts),
+// and each word counts its arrivals in its low 8 bits; a CTA polls the two
+// words until both counts are full and has the sum.  Integer addition makes
+// the sum independent of the order of arrival, and exact but for the parts'
+// truncations, less than one unit each: below 2^(8 - 72 + 10) = 2^-54 of the
+// smallest sum taken, a quarter of its last bit, before its rounding to double
+// precision.  (With a unit of 2^-67 and sums down to 2^-13 it was 2^-46.)
+// This replaces a store of the partial sum, the fence that publishes it, a
+// poll, a load of all partial sums and their additions: 5 100 -> 2 900 cycles
+// per sum with 152 CTAs.  A marked or unexpectedly small sum is taken again by
+// chip_sum, by every CTA alike.
 template <class F>
-__device__ __forceinline__ bool chip_sum_fast(GridSum& g, double v, double prev, F&& f) {
+__device__ __forceinline__ bool chip_sum_fast(GridSum& g, double v, double prev, F&& step) {
   const int t = threadIdx.x, lane = t & 31;
   const int ep = __double2hiint(prev) >> 20;  // sign and exponent
   const double v1[1] = {v};
-  if (ep < 256 || ep > 1790) return chip_sum<1>(g, v1, f);
+  if (ep < 256 || ep > 1790) return chip_sum<1>(g, v1, step);
   const unsigned G = gridDim.x;
   const int set = ++g.fast & 1;
   double s1[1];
   chip_cta_sum(g, v1, s1);
   if (t < 32) {
-    const long long bits = __double_as_longlong(s1[0]);
-    const int es = (int)(bits >> 52) & 0x7ff, sh = es - ep + 15;
-    const unsigned long long m = (bits & 0xfffffffffffffull) | (1ull << 52), low40 = (1ull << 40) - 1;
-    long long hi = 0;
-    unsigned long long lo = 0;
-    if (sh > 34) {
-      lo = 1ull << 48;  // out of range, inf or NaN
-    } else if (es > 0 && sh > -53) {
-      const unsigned long long w = sh < 0 ? m >> -sh : m;
-      const int up = sh < 0 ? 0 : sh;
-      lo = (w << up) & low40;
-      hi = (long long)(w >> (40 - up));
-      if (bits < 0) {
-        hi = lo ? -hi - 1 : -hi;
-        lo = (0 - lo) & low40;
-      }
-    }
+    const FixedParts f = fixed_parts(s1[0], ep);
     unsigned long long* word = g.sync->acc[set][lane & 1];
     unsigned long long* base = g.base + 2 * set + (lane & 1);
     unsigned long long w = 0;
     bool ok = true;
     if (lane < 2) {
-      const unsigned long long add = ((lane ? lo : (unsigned long long)hi) << 8) + 1ull;
+      const unsigned long long add = ((lane ? f.lo : (unsigned long long)f.hi) << 8) + 1ull;
       asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"(add) : "memory");
       const unsigned long long b0 = *base;
       long long t0 = 0;
@@ -212,19 +236,16 @@ __device__ __forceinline__ bool chip_sum_fast(GridSum& g, double v, double prev,
     ok = __all_sync(0xffffffffu, ok);
     const unsigned long long wlo = __shfl_sync(0xffffffffu, w, 1) >> 8;
     if (lane == 0) {
-      // the unit is 2^(ep - 1023 + 20 - 87); scaled by powers of two, exactly
-      const double unit = __longlong_as_double((long long)(ep - 67) << 52);
-      const double sum[1] = {fma((double)((long long)w >> 8), unit * 0x1p40, (double)(long long)wlo * unit)};
-      const int er = __double2hiint(sum[0]) >> 20;
-      const bool again = wlo >= (1ull << 48) || er < ep - 13;  // (a negative sum's er is negative)
+      bool again;
+      const double sum[1] = {fixed_value(FixedParts{(long long)w >> 8, wlo}, ep, again)};
       g.out[0] = sum[0];
       *g.ok = !ok ? 0 : again ? 2 : 1;
-      if (ok && !again) f(sum);
+      if (ok && !again) step(sum);
     }
   }
   __syncthreads();
   if (*g.ok != 2) return *g.ok != 0;
-  return chip_sum<1>(g, v1, f);
+  return chip_sum<1>(g, v1, step);
 }
 
 // What a solve does around its iterations: the double-precision solve from

@@ -4,6 +4,7 @@ from __future__ import annotations
 import ctypes
 import os
 import subprocess
+from fractions import Fraction
 
 import numpy as np
 
@@ -45,3 +46,55 @@ def dividends_and_divisors(n=1 << 20, seed=3):
 def same(a, b):
     """Equal bits, any NaN equal to any NaN."""
     return np.all((a.view(np.uint64) == b.view(np.uint64)) | (np.isnan(a) & np.isnan(b)))
+
+
+def sums(G, seed=5):
+    """(partial sums [cases, G], sums an iteration earlier [cases]): positive and mixed partial
+    sums whose total lies 2^-20 .. 2^18 from the earlier sum, one that
+    outweighs all others, zeros, the ends of the range, infinities and NaN."""
+    rng = np.random.default_rng(seed)
+    part, prev = [], []
+    for scale in (1.0, 3e-150, 7e140, 1e-290, 1e290, 5e-324, 0.0, -2.0, np.inf, np.nan):
+        for ratio in range(-20, 19):
+            for kind in range(3):
+                p = rng.uniform(0.0, 1.0, G)
+                if kind == 1:
+                    p[rng.random(G) < 0.5] *= -1.0
+                    p[0] = 2.0 * G  # the total stays positive
+                if kind == 2:
+                    p = p * 2.0 ** -rng.integers(0, 90, G)
+                    p[rng.integers(0, G)] = 1.0
+                with np.errstate(over="ignore", invalid="ignore", under="ignore"):
+                    base = scale if 1e-300 < scale < 1e300 else 1.0
+                    part.append(p / p.sum() * rng.uniform(0.6, 1.4) * 2.0 ** ratio * base)
+                prev.append(scale)
+    for special in (0.0, -1.0, np.inf, -np.inf, np.nan, 2.0 ** 40):
+        part.append(np.where(np.arange(G) == G // 2, special, 2.0 ** -30))
+        prev.append(1.0)
+    return np.array(part), np.array(prev)
+
+
+def check_sum(part, prev, got, retaken):
+    """The sum against the exact one.  A fixed-point sum is off by its
+    truncations, a quarter of its last bit, and the conversion's roundings: one
+    half (two where it exceeds 2^20 of the earlier sum).  A sum of doubles by
+    at most one rounding of the partial sums' total size per addition."""
+    if not np.all(np.isfinite(part)):
+        assert retaken
+        with np.errstate(invalid="ignore"):
+            want = part.sum()
+        assert np.isnan(got) if np.isnan(want) else got == want
+        return
+    total = sum(map(Fraction, part.tolist()))
+    error, exact = abs(Fraction(float(got)) - total), float(total)
+    if retaken:
+        assert error <= len(part) * Fraction(2) ** -53 * sum(map(Fraction, np.abs(part).tolist()))
+    else:
+        ulps = 0.25 + (0.5 if exact < 2.0 ** 20 * prev else 1.0)
+        assert error <= Fraction(ulps) * Fraction(float(np.spacing(exact))), (exact, prev)
+    # taken again or not, by the sums' size
+    if 1e-200 < prev < 1e200:
+        if 2.0 ** -9 * prev <= exact and max(abs(part)) < 2.0 ** 14 * prev:
+            assert not retaken
+        if exact < 2.0 ** -11 * prev or max(abs(part)) >= 2.0 ** 16 * prev:
+            assert retaken

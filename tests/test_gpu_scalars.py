@@ -1,5 +1,5 @@
-"""The solvers' scalar arithmetic (csrc/fp64.cuh) on the GPU against IEEE
-results: division and widening bit for bit, the finite, positive and
+"""The solvers' scalar arithmetic (csrc/fp64.cuh) and the on-chip solvers' grid
+sums (csrc/chip_solve.cuh) on the GPU against IEEE results and exact sums: division and widening bit for bit, the finite, positive and
 square-root tests by their outcome.  The square-root test may differ from
 sqrt(s) <= c only where both sides agree to 1e-12, and there it takes the exact
 test, so the outcomes are equal everywhere."""
@@ -67,3 +67,37 @@ def test_tests_of_a_sum(torch, lib):
     assert np.array_equal((out & 4) != 0, (out & 8) != 0)
     with np.errstate(invalid="ignore"):
         assert np.array_equal((out & 8) != 0, np.sqrt(s) <= c)
+
+
+def grid_sums(torch, lib, parts, prevs, absent=-1, timeout_ms=1000):
+    cases, G = parts.shape
+    out = torch.zeros((cases, G), dtype=torch.float64, device="cuda")
+    retaken = torch.full((cases, G), -1, dtype=torch.int32, device="cuda")
+    ok = torch.full((cases, G), -1, dtype=torch.int32, device="cuda")
+    status = np.zeros(1, np.int32)
+    a = [chip_check.addr(t) for t in (torch.from_numpy(parts).cuda(), torch.from_numpy(prevs).cuda(), out, retaken, ok)]
+    rc = lib.gpu_sums(*a, cases, G, absent, timeout_ms, chip_check.addr(status))
+    assert rc == 0
+    return out.cpu().numpy(), retaken.cpu().numpy(), ok.cpu().numpy(), int(status[0])
+
+
+@pytest.mark.parametrize("G", [1, 7, 152])
+def test_grid_sums(torch, lib, G):
+    parts, prevs = chip_check.sums(G)
+    out, retaken, ok, status = grid_sums(torch, lib, parts, prevs)
+    assert status == 0 and np.all(ok == 1)
+    for i in range(len(prevs)):
+        assert chip_check.same(out[i], np.full(G, out[i, 0])) and np.all(retaken[i] == retaken[i, 0])
+        if not 1e-200 < prevs[i] < 1e200:
+            assert retaken[i, 0] == 1  # the earlier sum's exponent is out of the fixed point's range
+        chip_check.check_sum(parts[i], prevs[i], out[i, 0], retaken[i, 0] == 1)
+
+
+@pytest.mark.parametrize("prev", [1.0, 0.0])
+def test_a_grid_sums_wait_ends(torch, lib, prev):
+    # a CTA that never arrives: both forms of the sum give up within their limit
+    _, _, ok, status = grid_sums(torch, lib, np.ones((1, 5)), np.array([prev]), absent=0, timeout_ms=20)
+    assert status == 5 and list(ok[0]) == [-1, 0, 0, 0, 0]
+    # and the device is as before
+    out, _, ok, status = grid_sums(torch, lib, np.ones((1, 5)), np.array([prev]))
+    assert status == 0 and np.all(ok == 1) and np.all(out == 5.0)
