@@ -461,9 +461,12 @@ cudaError_t launch_cg_fmt(const gbcg_matrix_s* M, const CgArgs<V>& a, cudaStream
 }
 
 template <int FMT>
-cudaError_t launch_pcg(const PcgArgs<double>& args, int grid, cudaStream_t s) {
+cudaError_t launch_pcg(const gbcg_matrix_s* M, const PcgArgs<double>& args, cudaStream_t s) {
   void* kargs[] = {(void*)&args};
-  return cudaLaunchCooperativeKernel((const void*)k_pcg<double, FMT>, dim3(grid), dim3(block_of(FMT)), kargs,
+  // by diagonals a thread owns rows, and warps without any would only add
+  // their zeros to the CTA's sums, 5 FP64 instructions each and sum
+  const int threads = is_dia(FMT) ? (int)std::min<int64_t>(block_of(FMT), M->chip_rows) : block_of(FMT);
+  return cudaLaunchCooperativeKernel((const void*)k_pcg<double, FMT>, dim3(M->grid), dim3(threads), kargs,
                                      product_smem<double, FMT>(), s);
 }
 
@@ -476,9 +479,9 @@ cudaError_t launch_pcg_fmt(const gbcg_matrix_s* M, const CgArgs<double>& c, cuda
   a.z = M->z64;
   a.w0 = M->w64a;
   a.w1 = M->w64b;
-  return M->mode == kPlan  ? launch_pcg<kPlan>(a, M->grid, s)
-         : M->mode == kDia ? launch_pcg<kDia>(a, M->grid, s)
-                           : launch_pcg<kGather>(a, M->grid, s);
+  return M->mode == kPlan  ? launch_pcg<kPlan>(M, a, s)
+         : M->mode == kDia ? launch_pcg<kDia>(M, a, s)
+                           : launch_pcg<kGather>(M, a, s);
 }
 
 template <int FMT>
