@@ -216,6 +216,8 @@ struct gbcg_matrix_s {
   std::vector<int32_t> h_ptr, h_idx;
   int32_t *u_map_main = nullptr, *u_map_long = nullptr, *u_map_diag = nullptr;
   int64_t u_len_main = 0, u_len_long = 0, u_len_diag = 0;
+  uint8_t* u_slot = nullptr;   // diagonal layout: places within the lines, and the lines' starts
+  int32_t* u_ptr = nullptr;
   double* u_stage = nullptr;
   int64_t nslices = 0, nlong = 0, bytes = 0;
   int sym = 0;
@@ -346,7 +348,7 @@ void free_matrix(gbcg_matrix_s* M) {
                  M->long_val64, M->long_val32, M->diag64, M->diag32, M->pl_ptr, M->pl_i, M->pl_k,
                  M->cta_slice, M->cta_long, M->r, M->p_base, M->q, M->bstage, M->xstage, M->r32, M->p32_base, M->q32,
                  M->d32, M->rhs32, M->part, M->sums, M->sync, M->st, M->u_map_main, M->u_map_long, M->u_map_diag,
-                 M->u_map_t32, M->u_stage, M->dia64, M->dia32, M->s64, M->z64, M->w64a, M->w64b};
+                 M->u_map_t32, M->u_slot, M->u_ptr, M->u_stage, M->dia64, M->dia32, M->s64, M->z64, M->w64a, M->w64b};
   M->t32.release();
   M->t64.release();
   for (void* d : dev)
@@ -1216,19 +1218,22 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
   if (nnz == 0) return GBCG_OK;
   if (!val) return fail(GBCG_ERR_INVALID, "null value array");
   cudaStream_t s = (cudaStream_t)stream;
-  if (!A->u_map_main && !A->u_map_long && !A->u_map_diag) {
+  if (is_dia(A->mode)) {
+    if (!A->u_slot) {
+      std::vector<uint8_t> slots;
+      diagonal_slots(A->format, A->n, A->h_ptr.data(), A->h_idx.data(), A->index_base, A->dia_off, slots);
+      if (int rc = upload(&A->u_ptr, A->h_ptr, s, A->bytes)) return rc;
+      if (int rc = upload(&A->u_slot, slots, s, A->bytes)) return rc;
+      if (int rc = dalloc(&A->u_stage, (size_t)nnz, A->bytes)) return rc;
+    }
+  } else if (!A->u_map_main && !A->u_map_long && !A->u_map_diag) {
     // the layout of the same pattern with value k + 1 at input entry k: every
     // device value slot then names the input entry it holds (0: padding)
     std::vector<double> iv(nnz);
     for (int64_t k = 0; k < nnz; ++k) iv[k] = (double)(k + 1);
-    const bool diagonals = A->mode == kDia || A->mode == kDiaSym;
     LayoutHost L;
-    DiaHost Dh;
     std::string err;
-    if (diagonals) {
-      if (!build_diagonals(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, Dh))
-        return fail(GBCG_ERR_INVALID, "rebuilding the value map: diagonals differ from the handle's");
-    } else if (A->sym && A->mode == kGather) {
+    if (A->sym && A->mode == kGather) {
       if (!build_sym_full(A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, L))
         return fail(GBCG_ERR_INVALID, "rebuilding the value map: layout differs from the handle's");
     } else if (int rc = build_layout(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base,
@@ -1253,9 +1258,6 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
       A->u_len_main = (int64_t)T64.val.size();
       if (int rc = upload(&A->u_map_t32, to_map(T32.val), s, B)) return rc;
       A->u_len_t32 = (int64_t)T32.val.size();
-    } else if (diagonals) {
-      if (int rc = upload(&A->u_map_main, to_map(Dh.val), s, B)) return rc;
-      A->u_len_main = (int64_t)Dh.val.size();
     } else {
       if (int rc = upload(&A->u_map_main, to_map(L.A.val), s, B)) return rc;
       A->u_len_main = (int64_t)L.A.val.size();
@@ -1264,7 +1266,7 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
         A->u_len_long = (int64_t)L.A.long_val.size();
       }
     }
-    if (A->sym && !diagonals && A->mode != kGather) {
+    if (A->diag64) {
       if (int rc = upload(&A->u_map_diag, to_map(L.diag), s, B)) return rc;
       A->u_len_diag = (int64_t)L.diag.size();
     }
@@ -1278,15 +1280,18 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
   auto run = [&](const int32_t* map, int64_t len, double* d64, float* d32) -> int {
     if (!map || len == 0) return 0;
     const int blocks = (int)std::min<int64_t>(4096, (len + 255) / 256);
-    k_place_values<<<blocks, 256, 0, s>>>(map, len, src, d64, d32, A->mode == kDia || A->mode == kDiaSym);
+    k_place_values<<<blocks, 256, 0, s>>>(map, len, src, d64, d32);
     CUDA_TRY(cudaGetLastError());
     return 0;
   };
   if (A->mode == kTiles) {
     if (int rc = run(A->u_map_main, A->u_len_main, (double*)A->t64.val, nullptr)) return rc;
     if (int rc = run(A->u_map_t32, A->u_len_t32, nullptr, (float*)A->t32.val)) return rc;
-  } else if (A->mode == kDia || A->mode == kDiaSym) {
-    if (int rc = run(A->u_map_main, A->u_len_main, A->dia64, A->dia32)) return rc;
+  } else if (is_dia(A->mode)) {
+    const int blocks = (int)std::min<int64_t>(4096, A->nslices * ((int64_t)A->dia_off.size() + 2) / 3 / 8 + 1);
+    k_place_diagonals<<<blocks, kPlaceThreads, 0, s>>>(A->dia<double>(), A->format == GBCG_CSC, A->u_ptr,
+                                                       A->index_base, A->u_slot, src, A->dia64, A->dia32);
+    CUDA_TRY(cudaGetLastError());
   } else {
     if (int rc = run(A->u_map_main, A->u_len_main, A->val64, A->val32)) return rc;
     if (int rc = run(A->u_map_long, A->u_len_long, A->long_val64, A->long_val32)) return rc;

@@ -131,6 +131,21 @@ bool build_diagonals(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr,
   return true;
 }
 
+void diagonal_slots(int32_t format, int64_t n, const int32_t* ptr, const int32_t* idx, int32_t base,
+                    const std::vector<int32_t>& off, std::vector<uint8_t>& out) {
+  out.assign(off.size() * (size_t)n, kNoSlot);
+  for (int64_t r = 0; r < n; ++r) {
+    const int64_t k0 = (int64_t)ptr[r] - base, len = (int64_t)ptr[r + 1] - base - k0;
+    size_t at = 0;
+    for (int64_t m = 0; m < len; ++m) {
+      const int64_t j = format == 2 ? len - 1 - m : m;  // a column's offsets (column - row) decrease
+      const int64_t o = (int64_t)idx[k0 + j] - base - r;
+      while (off[at] != (format == 2 ? -o : o)) ++at;
+      out[at * (size_t)n + r] = (uint8_t)j;
+    }
+  }
+}
+
 namespace {
 
 // Slices rows into the SELL-32 layout; rows longer than `long_threshold` go

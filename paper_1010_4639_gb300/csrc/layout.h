@@ -173,6 +173,13 @@ int validate_input(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, c
 bool build_diagonals(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                      const double* val, int32_t index_base, DiaHost& out);
 
+// Where the entries of a validated input that has the diagonals `off` lie
+// within their lines: out[k * n + line] is the place of the entry on diagonal k
+// among the line's entries, kNoSlot where there is none.
+constexpr uint8_t kNoSlot = 255;
+void diagonal_slots(int32_t format, int64_t n, const int32_t* ptr, const int32_t* idx, int32_t index_base,
+                    const std::vector<int32_t>& off, std::vector<uint8_t>& out);
+
 // Windows of a tile's rows (480; fewer in a small matrix) of a validated
 // symmetric input, per tile on average: runs of consecutive rows beyond the
 // block that its upper entries reach.  Three or four for a mesh numbered line
