@@ -230,9 +230,16 @@ __device__ __forceinline__ void dia_segment(const E& entry, int K, int lo, int h
     if (!dia_finite(acc[r])) acc[r] = dia_row_exact<SYM, NC>(entry, K, val, n, min(i0 + 32 * r, last), x);
 }
 
+// Diagonals in flight, for K of them: chunks of eight would read one or two
+// diagonals eight times over (2.0 M rows, symmetric, two stored diagonals,
+// double precision: 58 us for a product in chunks of eight, 19 in chunks of two,
+// tiles 41; three stored diagonals 58, 31 and 49).  Chosen once per product: at
+// the end of every row's diagonals it cost the 15-diagonal products 1-3%.
+__host__ __device__ constexpr int dia_few(int K) { return K <= 2 ? 2 : K <= 4 ? 4 : 8; }
+
 // f(row, (A x)_row) for the rows [r0, r1) of the CTA.
 template <bool SYM, bool HALO, int C, int R, typename V, class F>
-__device__ __forceinline__ void dia_rows(const DiaTab<V>& t, int r0, int r1, const V* x, F&& f) {
+__device__ __forceinline__ void dia_rows_in(const DiaTab<V>& t, int r0, int r1, const V* x, F&& f) {
   const int lane = threadIdx.x & 31, step = blockDim.x * R;
   for (int base = r0 + (threadIdx.x >> 5) * 32 * R; base < r1; base += step) {
     V acc[R];
@@ -241,6 +248,14 @@ __device__ __forceinline__ void dia_rows(const DiaTab<V>& t, int r0, int r1, con
     for (int r = 0; r < R; ++r)
       if (base + lane + 32 * r < r1) f(base + lane + 32 * r, acc[r]);
   }
+}
+template <bool SYM, bool HALO, int C, int R, typename V, class F>
+__device__ __forceinline__ void dia_rows(const DiaTab<V>& t, int r0, int r1, const V* x, F&& f) {
+  if constexpr (C == 8) {
+    if (dia_few(t.K) == 2) return dia_rows_in<SYM, HALO, 2, R>(t, r0, r1, x, f);
+    if (dia_few(t.K) == 4) return dia_rows_in<SYM, HALO, 4, R>(t, r0, r1, x, f);
+  }
+  dia_rows_in<SYM, HALO, C, R>(t, r0, r1, x, f);
 }
 
 // Product of the solvers whose vectors stay in global memory: rows per thread
@@ -291,14 +306,14 @@ __device__ __forceinline__ V dia_sweep(const DiaTab<V>& t, int64_t r0, int64_t r
   return dot;
 }
 
-// y = A x, R rows per thread.
-template <typename V, bool SYM, int R>
+// y = A x, R rows per thread, C diagonals in flight.
+template <typename V, bool SYM, int R, int C>
 __global__ void __launch_bounds__(kDiaBlock) k_dia_rows(const __grid_constant__ DiaDev<V> A, const V* __restrict__ x,
                                                        V* __restrict__ y) {
   const int base = (int)((blockIdx.x * (kDiaBlock / 32) + (threadIdx.x >> 5)) * 32 * R), n = (int)A.n;
   if (base >= n) return;
   V acc[R];
-  dia_segment<SYM, true, false, R == 1 ? 8 : 4, R>(DiaParam<V>{A}, A.K, A.lo, A.hi, A.val, n, n - 1, base, x, acc);
+  dia_segment<SYM, true, false, C, R>(DiaParam<V>{A}, A.K, A.lo, A.hi, A.val, n, n - 1, base, x, acc);
   const int i0 = base + (threadIdx.x & 31);
 #pragma unroll
   for (int r = 0; r < R; ++r)

@@ -555,10 +555,16 @@ cudaError_t launch_product(const gbcg_matrix_s* M, const V* x, const V* b, V* y,
     // pipe's queue (128^3: 60 us against 120 with two)
     constexpr int R = dia_r<V>();
     auto blocks = [&](int rows) { return (unsigned)((M->n + rows * kDiaBlock - 1) / (rows * kDiaBlock)); };
-    if (M->n > 300000)
-      k_dia_rows<V, FMT == kDiaSym, R><<<blocks(R), kDiaBlock, 0, s>>>(M->dia<V>(), x, y);
+    constexpr bool S = FMT == kDiaSym;
+    const DiaDev<V> D = M->dia<V>();
+    if (R > 1 && M->n > 300000)
+      k_dia_rows<V, S, R, 4><<<blocks(R), kDiaBlock, 0, s>>>(D, x, y);
+    else if (dia_few(D.K) == 2)
+      k_dia_rows<V, S, 1, 2><<<blocks(1), kDiaBlock, 0, s>>>(D, x, y);
+    else if (dia_few(D.K) == 4)
+      k_dia_rows<V, S, 1, 4><<<blocks(1), kDiaBlock, 0, s>>>(D, x, y);
     else
-      k_dia_rows<V, FMT == kDiaSym, 1><<<blocks(1), kDiaBlock, 0, s>>>(M->dia<V>(), x, y);
+      k_dia_rows<V, S, 1, 8><<<blocks(1), kDiaBlock, 0, s>>>(D, x, y);
   } else
     k_rows<V, FMT><<<M->grid, block_of(FMT), product_smem<V, FMT>(), s>>>(
       M->op<V>(), M->tiles<V>(), M->cta_slice, M->cta_long, x, y, &M->bar->status, 1000000000LL);
