@@ -91,6 +91,17 @@ struct BDia {
   int32_t ld, K;
   int32_t off[gbcg::kMaxDiag];
 };
+// Largest instance by diagonals: its values and the direction's eight columns,
+// in bytes.  Split over a cluster of 16 they stay in the CTAs' L1 up to about
+// 3.3 MB; beyond, the diagonals' 64-byte pieces per warp cost more than CSR's
+// rows.  Equal cubes of 15 diagonals, reliable updates, 300 iterations, ms by
+// diagonals / in CSR: 32 768 rows (3.0 MB) 8 systems 12.0 / 13.8, 40 systems
+// 40.6 / 44.1; 46 656 rows (4.3 MB) 8 systems 16.9 / 18.8, 40 systems 68.1 /
+// 62.9; 54 872 rows (5.0 MB) 40 systems 84.3 / 76.4; 97 336 rows 8 systems 42.3
+// / 39.3.  Where the two cross depends on how many run together; the line keeps
+// the small batches' gain (48 uneven systems of up to 54 872 rows: 63.0 ms, 64.8
+// with the line at 3.3 MB).
+constexpr int64_t kDiaInstanceBytes = 4500000;
 
 // Everything a launch reads, kept in device memory so that a captured graph
 // serves every solve (the host rewrites this block before each launch).
@@ -936,7 +947,6 @@ __device__ bool solve_instance_ru(const BArgs& a, const BDia& dia, int inst, Gro
       };
       if (dia.K > 0) product_dia(dia, a.dia32, P, row0, (int)nI, r0, r1, emit);
       else product_rpw<float>(rp, a.ptr, a.idx, a.val32, P, r0, r1, emit);
-      double v[1][VW];
       const double s = group_reduce1<NT>(a, pq, red, par, g, s_flag, ok);
       if (!ok) return false;
       if (t < 32) {
@@ -1690,12 +1700,14 @@ int gbcg_batch_create(gbcg_batch_t* out, int32_t count, const int64_t* row_off, 
     std::vector<int32_t> lp, li;
     for (int i = 0; i < count; ++i) {
       const int64_t r0 = row_off[i], m = row_off[i + 1] - r0, z = B->nnz_of[i], k0 = ptr[r0];
+      if (m * (int64_t)(sizeof(float) * (1 + kRhs)) > kDiaInstanceBytes) continue;
       lp.resize(m + 1);
       li.resize(z);
       for (int64_t r = 0; r <= m; ++r) lp[r] = (int32_t)(ptr[r0 + r] - k0);
       for (int64_t k = 0; k < z; ++k) li[k] = (int32_t)(idx[k0 + k] - r0);
       gbcg::DiaHost H;
-      if (!gbcg::build_diagonals(GBCG_CSR, m, z, lp.data(), li.data(), val + k0, 0, H) || H.ld * (int64_t)H.off.size() > 0x7fffffff)
+      if (!gbcg::build_diagonals(GBCG_CSR, m, z, lp.data(), li.data(), val + k0, 0, H) ||
+          m * (int64_t)(sizeof(float) * (H.off.size() + kRhs)) > kDiaInstanceBytes)
         continue;
       dia[i].base = (int64_t)dval.size();
       dia[i].ld = (int32_t)H.ld;
@@ -1706,7 +1718,8 @@ int gbcg_batch_create(gbcg_batch_t* out, int32_t count, const int64_t* row_off, 
   }
   const size_t nv = (size_t)std::max<int64_t>(1, n) * kRhs;
   int rc = 0;
-  if ((rc = balloc(B, &B->d_dia, count)) || (rc = balloc(B, &B->d_dia32, dval.size())) || (rc = balloc(B, &B->d_inst_row, count + 1)) || (rc = balloc(B, &B->d_ptr, n + 1)) ||
+  if ((rc = balloc(B, &B->d_dia, count)) || (rc = balloc(B, &B->d_dia32, dval.size())) ||
+      (rc = balloc(B, &B->d_inst_row, count + 1)) || (rc = balloc(B, &B->d_ptr, n + 1)) ||
       (rc = balloc(B, &B->d_idx, nnz)) || (rc = balloc(B, &B->d_val64, nnz)) || (rc = balloc(B, &B->d_val32, nnz)) ||
       (rc = balloc(B, &B->d_slot_inst, (size_t)count * kMaxGroup)) ||
       (rc = balloc(B, &B->d_slot_part, (size_t)count * kMaxGroup)) || (rc = balloc(B, &B->d_grp, count)) ||

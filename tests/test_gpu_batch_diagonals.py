@@ -1,0 +1,52 @@
+"""Which instances of a small batch are computed by diagonals: instances on
+either side of the size limit solve to the same tolerance, and a batch of large
+instances is not slower for having diagonals."""
+import numpy as np
+import pytest
+
+import femgen
+import paper_1010_4639_gb300 as gb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch
+    gb.build()
+    assert torch.cuda.is_available()
+    return torch
+
+
+@pytest.mark.parametrize("precision", ["fp32_ru", "fp32_ir"])
+def test_instances_around_the_limit(torch, precision):
+    # 15 diagonals: the limit lies between 47 952 and 49 248 rows
+    bs = femgen.build_batch([femgen.Grid(*g, contrast=10.0, jitter=0.15)
+                             for g in ((38, 38, 39), (38, 38, 40), (9, 9, 9))], nrhs=8)
+    with gb.Batch(bs.row_off, bs.ptr, bs.idx, bs.val, nrhs=8, tune=False) as B:
+        x, infos, rep = B.solve(torch.from_numpy(bs.B).cuda(), tol=1e-12, maxit=20000, precision=precision)
+    assert rep["status"] == "OK"
+    import oracle
+    x = x.cpu().numpy()
+    for i in range(bs.count):
+        p, j, v = bs.instance(i)
+        a, z = bs.row_off[i], bs.row_off[i + 1]
+        for k in range(8):
+            r = bs.B[a:z, k] - oracle.spmv("csr", p, j, v, np.ascontiguousarray(x[a:z, k]))
+            assert np.linalg.norm(r) <= 1.001e-12 * np.linalg.norm(bs.B[a:z, k])
+
+
+def test_large_instances_are_not_slower_by_diagonals(torch, monkeypatch):
+    # 40 cubes of 54 872 rows, refinement, the same tuned launch for both (the
+    # second batch takes the first one's table): all by diagonals 86 ms, in CSR
+    # 77.  A twentieth is allowed for what runs differ by
+    bs = femgen.build_batch([femgen.Grid(40, 40, 40, contrast=10.0, jitter=0.15)] * 40, nrhs=8)
+    b = torch.from_numpy(bs.B).cuda()
+    best = {}
+    for flag in ("1", "0"):
+        monkeypatch.setenv("GBCG_DIAGONALS", flag)
+        with gb.Batch(bs.row_off, bs.ptr, bs.idx, bs.val, nrhs=8) as B:
+            times = [B.solve(b, tol=1e-13, maxit=300, precision="fp32_ir", raise_on_error=False)[2]["kernel_ms"]
+                     for _ in range(6)]
+            best[flag] = min(times)
+    assert best["1"] <= 1.05 * best["0"], best
