@@ -1205,6 +1205,7 @@ struct gbcg_batch_s {
   double* d_val64 = nullptr;
   float* d_val32 = nullptr;
   BDia* d_dia = nullptr;
+  int ndia = 0;  // instances by diagonals
   float* d_dia32 = nullptr;
   int8_t* d_rpw = nullptr;
   double* d_R64 = nullptr;
@@ -1300,6 +1301,8 @@ std::string tune_key(const gbcg_batch_s* B, bool f32) {
   k += "|n" + std::to_string(lg((double)B->n_tot)) + "|z" + std::to_string(lg((double)B->nnz_tot)) + "|c" +
        std::to_string(lg((double)B->count)) + "|r" + std::to_string(B->nrhs);
   for (int b = 0; b < kBuckets; ++b) k += "|" + std::to_string(lg((double)hist[b]));
+  // systems by diagonals (single-precision forms): their launch configuration is another one's
+  if (f32) k += "|d" + std::to_string(B->ndia ? 1 + lg((double)B->ndia) : 0);
   return k;
 }
 
@@ -1709,6 +1712,7 @@ int gbcg_batch_create(gbcg_batch_t* out, int32_t count, const int64_t* row_off, 
       if (!gbcg::build_diagonals(GBCG_CSR, m, z, lp.data(), li.data(), val + k0, 0, H) ||
           m * (int64_t)(sizeof(float) * (H.off.size() + kRhs)) > kDiaInstanceBytes)
         continue;
+      ++B->ndia;
       dia[i].base = (int64_t)dval.size();
       dia[i].ld = (int32_t)H.ld;
       dia[i].K = (int32_t)H.off.size();

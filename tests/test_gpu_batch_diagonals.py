@@ -50,3 +50,14 @@ def test_large_instances_are_not_slower_by_diagonals(torch, monkeypatch):
                      for _ in range(6)]
             best[flag] = min(times)
     assert best["1"] <= 1.05 * best["0"], best
+
+
+def test_tuning_of_a_batch_by_diagonals_is_its_own(torch, monkeypatch):
+    # the same sizes with and without diagonals: the second batch is not given the first one's launch
+    bs = femgen.build_batch([femgen.Grid(11, 12, 13, contrast=10.0, jitter=0.15)] * 3, nrhs=8)
+    cached = []
+    for flag in ("1", "0", "1", "0"):
+        monkeypatch.setenv("GBCG_DIAGONALS", flag)
+        with gb.Batch(bs.row_off, bs.ptr, bs.idx, bs.val, nrhs=8, tune=False) as B:
+            cached.append(B.autotune("fp32_ir")["from_cache"])
+    assert cached == [0, 0, 1, 1]
