@@ -924,7 +924,7 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
                         sym_windows(n, ptr, idx, index_base) > kTileWindows &&
                         sym_slices_fit(n, ptr, idx, index_base, TileCaps<double>::kSlot, TileCaps<double>::kEnt) &&
                         build_sym_full(n, nnz, ptr, idx, val, index_base, L);
-  if (!diagonals && !sym_full && (rc = build_layout(format, n, nnz, ptr, idx, val, index_base, L, err)) != 0)
+  if (!diagonals && !sym_full && (rc = build_rows(format, n, nnz, ptr, idx, val, index_base, L, err)) != 0)
     return fail(rc, err);
   // debug mode: full CSR/CSC inputs must be symmetric (CG's premise)
   if (format != GBCG_SYM_CSR_UPPER && env_int("GBCG_CHECK_SYMMETRY", 0) != 0 &&
@@ -1242,8 +1242,8 @@ int gbcg_update_values(gbcg_matrix_t A, const double* val, int32_t memory, void*
     if (A->sym && A->mode == kGather) {
       if (!build_sym_full(A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base, L))
         return fail(GBCG_ERR_INVALID, "rebuilding the value map: layout differs from the handle's");
-    } else if (int rc = build_layout(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base,
-                                     L, err)) {
+    } else if (int rc = build_rows(A->format, A->n, nnz, A->h_ptr.data(), A->h_idx.data(), iv.data(), A->index_base,
+                                   L, err)) {
       return fail(rc, "rebuilding the value map: " + err);
     }
     SymTilesHost T32, T64;

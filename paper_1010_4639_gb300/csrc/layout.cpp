@@ -325,8 +325,12 @@ bool build_sym_full(int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* i
 
 int build_layout(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                  const double* val, int32_t base, LayoutHost& out, std::string& err) {
-  int rc = validate_input(format, n, nnz, ptr, idx, val, base, err);
-  if (rc) return rc;
+  if (int rc = validate_input(format, n, nnz, ptr, idx, val, base, err)) return rc;
+  return build_rows(format, n, nnz, ptr, idx, val, base, out, err);
+}
+
+int build_rows(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
+               int32_t base, LayoutHost& out, std::string& err) {
   out = LayoutHost();
   out.format = format;
   out.n = n;

@@ -197,8 +197,12 @@ bool sym_slices_fit(int64_t n, const int32_t* ptr, const int32_t* idx, int32_t i
 bool build_sym_full(int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
                     int32_t index_base, LayoutHost& out);
 
-// Validates the input and builds the row-gather (or symmetric) layout.
-// Returns 0 or a gbcg_status error code, with a message in `err`.
+// Builds the row-gather (or symmetric) layout of a validated input.  Returns 0
+// or a gbcg_status error code, with a message in `err`.
+int build_rows(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx, const double* val,
+               int32_t index_base, LayoutHost& out, std::string& err);
+
+// The same, validating the input first.
 int build_layout(int32_t format, int64_t n, int64_t nnz, const int32_t* ptr, const int32_t* idx,
                  const double* val, int32_t index_base, LayoutHost& out, std::string& err);
 
