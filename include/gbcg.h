@@ -121,8 +121,11 @@ typedef struct {
   int64_t plan_slots;         /* SELL slots of the symmetric transpose plan (0 if none) */
   int64_t long_rows;          /* rows handled warp-per-row */
   int64_t device_bytes;       /* device memory held by the handle */
-  int64_t spmv_bytes_fp64;    /* algorithmic bytes of one double-precision product (value +
-                                 index per entry, row pointers, x read once, y written once) */
+  int64_t spmv_bytes_fp64;    /* bytes one double-precision product needs in its layout: by
+                                 diagonals the values of their rows; by rows value + index of
+                                 every entry multiplied (symmetric storage: both copies) and row
+                                 pointers; by tiles or plan value + 4-byte index of every stored
+                                 entry and row pointers; x read once, y written once */
   int64_t spmv_bytes_fp32;    /* the same for the single-precision product */
   int64_t ext_slots;          /* symmetric tiles: partial sums leaving the tiles */
   int32_t format;             /* gbcg_format */
@@ -132,11 +135,13 @@ typedef struct {
                                  (tiles, diagonals, or the full operator's rows where the numbering
                                  scatters the neighbours) */
   int32_t tiles;              /* symmetric tiles: number of tiles (0 in the other layouts) */
-  int32_t index_bytes;        /* bytes per column index in the product's stream: 2 when the
-                                 row-gather layout stores 16-bit offsets from the row (every
-                                 offset fits; natural-order finite-element matrices up to
-                                 about 180^3 nodes), else 4 */
-  int32_t pad_;
+  int32_t index_bytes;        /* bytes per column index of the matrix by rows: 2 when every
+                                 offset from the row fits 16 bits (natural-order finite-element
+                                 matrices up to about 180^3 nodes; full storage, or symmetric
+                                 storage computed by rows), else 4.  By diagonals (product 3, 4) no
+                                 index is stored */
+  int32_t product;            /* layout the product runs on: 0 rows, 1 transpose plan, 2 tiles,
+                                 3 diagonals, 4 diagonals of the upper half */
 } gbcg_matrix_stats;
 
 /*

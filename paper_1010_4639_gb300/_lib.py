@@ -51,7 +51,7 @@ class Stats(ctypes.Structure):
                 ("device_bytes", ctypes.c_int64), ("spmv_bytes_fp64", ctypes.c_int64),
                 ("spmv_bytes_fp32", ctypes.c_int64), ("ext_slots", ctypes.c_int64), ("format", ctypes.c_int32),
                 ("grid_ctas", ctypes.c_int32), ("layout", ctypes.c_int32), ("tiles", ctypes.c_int32),
-                ("index_bytes", ctypes.c_int32), ("pad_", ctypes.c_int32)]
+                ("index_bytes", ctypes.c_int32), ("product", ctypes.c_int32)]
 
 
 class BatchInfo(ctypes.Structure):

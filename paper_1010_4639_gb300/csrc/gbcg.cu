@@ -1201,12 +1201,16 @@ int gbcg_stats(gbcg_matrix_t A, gbcg_matrix_stats* out) {
   out->plan_slots = A->plan_slots;
   out->long_rows = A->nlong;
   out->device_bytes = A->bytes;
-  const int64_t n = A->n, m = A->nnz_input;
-  // the product's matrix stream: value + column index per entry (2-byte
-  // offsets in the row-gather layout when they fit), row pointers, x, y
-  const int64_t ib = A->narrow && !A->sym ? 2 : 4;
-  out->spmv_bytes_fp64 = (8 + ib) * m + 4 * (n + 1) + 16 * n;
-  out->spmv_bytes_fp32 = (4 + ib) * m + 4 * (n + 1) + 8 * n;
+  const int64_t n = A->n, ib = A->narrow && (!A->sym || A->mode == kGather) ? 2 : 4;
+  // the matrix stream of a product with values of v bytes
+  auto matrix_bytes = [&](int64_t v) -> int64_t {
+    if (is_dia(A->mode)) return v * (int64_t)A->dia_off.size() * n;
+    if (A->mode == kGather) return (v + ib) * A->nnz_full + 4 * (n + 1);
+    return (v + 4) * A->nnz_input + 4 * (n + 1);
+  };
+  out->spmv_bytes_fp64 = matrix_bytes(8) + 16 * n;
+  out->spmv_bytes_fp32 = matrix_bytes(4) + 8 * n;
+  out->product = A->mode;
   out->index_bytes = (int32_t)ib;
   out->format = A->format;
   out->grid_ctas = A->grid;
