@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(kGradThreads) k_assemble(int64_t nnz, const in
     // a counting sort by number of contributions (ties in any order: it only
     // decides which thread sums which position)
     const int64_t n0 = t < cnt ? ptr[t + 1] - ptr[t] : 0;
-    const int b = n0 < kBins ? (int)n0 : kBins - 1;
+    // (a decreasing pointer is a position without contributions)
+    const int b = n0 < 0 ? 0 : n0 < kBins ? (int)n0 : kBins - 1;
     const int rank = t < cnt ? atomicAdd(&bin[b], 1) : 0;
     __syncthreads();
     if (t < kBins) {
