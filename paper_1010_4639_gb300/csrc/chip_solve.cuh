@@ -443,7 +443,11 @@ __global__ void __launch_bounds__(chip_threads(R), 1) k_cg_chip(const __grid_con
     at_delta.set(a.delta * rmax);
     return true;
   };
-  // p = r + beta p of the CTA's rows, on the chip and out
+  // p = r + beta p of the CTA's rows, on the chip and out.  Another CTA may have
+  // read the former p as the two sums since then order nothing in memory; but
+  // what it read went into its part of p'q, which it could only publish once
+  // the values were there, and this CTA has waited for every part.  (Reads
+  // whose value is not used may see either p.)
   auto direction = [&]() -> bool {
     const V be = (V)beta;
     for (int i = r0 + t; i < r1; i += T) {

@@ -84,8 +84,12 @@ constexpr int kTileSlices32 = kTileWarps * TileCaps<float>::kRpt, kTileSlices64 
 // Windows per tile (layout.h, sym_windows) up to which symmetric storage
 // is computed by tiles.  Twice what a tile's descriptor holds; a mesh numbered
 // line by line has 3 or 4, one renumbered at random within 2048 unknowns some
-// 100, where a reliable-update iteration of 85 000 rows took 435 us in tiles
-// and takes 9 with the full operator's row gather.
+// 100.  us per reliable-update iteration, tiles / the full operator's row
+// gather: 85 000 rows, 100 windows 435 / 9; 0.65 M rows, 19 windows 94 / 32,
+// 102 windows 588 / 34; 2.0 M rows, 23 windows 246 / 70, 99 windows 1 558 / 75;
+// 5.1 M rows, 18 windows 418 / 175.  Below the line the tiles hold half the
+// bytes and are the faster form on large systems with few windows only (2.0 M
+// rows, 2 windows 55 / 60, 4 windows 90 / 60; 5.1 M rows, 2.5 windows 131 / 151).
 constexpr double kTileWindows = 2 * kDescWin;
 
 int env_int(const char* name, int dflt) {
@@ -739,13 +743,14 @@ cudaError_t enqueue_ru(gbcg_matrix_s* M, const double* b, double* x, double tol,
     ca.maxit = maxit;
     ca.timeout_ns = a.c.timeout_ns;
     e = launch_chip_fmt<float, kSolveRu>(M, ca, s);
-  } else
-  switch (M->mode) {
-    case kTiles: e = launch_ru<kTiles>(a, M->grid, s); break;
-    case kPlan: e = launch_ru<kPlan>(a, M->grid, s); break;
-    case kDia: e = launch_ru<kDia>(a, M->grid, s); break;
-    case kDiaSym: e = launch_ru<kDiaSym>(a, M->grid, s); break;
-    default: e = launch_ru<kGather>(a, M->grid, s); break;
+  } else {
+    switch (M->mode) {
+      case kTiles: e = launch_ru<kTiles>(a, M->grid, s); break;
+      case kPlan: e = launch_ru<kPlan>(a, M->grid, s); break;
+      case kDia: e = launch_ru<kDia>(a, M->grid, s); break;
+      case kDiaSym: e = launch_ru<kDiaSym>(a, M->grid, s); break;
+      default: e = launch_ru<kGather>(a, M->grid, s); break;
+    }
   }
   if (e != cudaSuccess) return e;
   return timed ? cudaEventRecord(M->ev1, s) : cudaSuccess;
@@ -827,7 +832,7 @@ int solve_ir(gbcg_matrix_s* M, const double* b, double* x, double tol, int maxit
         ChipArgs<float> ca = {};
         ca.x = M->d32;
         ca.b = M->rhs32;
-            ca.p = M->p32;
+        ca.p = M->p32;
         ca.tol = inner_tol;
         ca.maxit = maxit - used;
         ca.timeout_ns = tns;
@@ -963,7 +968,12 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
     return bail(fail(GBCG_ERR_CUDA, "cannot query the device"));
   M->l2_bytes = l2;
-  M->mode = diagonals ? (M->sym ? kDiaSym : kDia) : !M->sym || sym_full ? kGather : (sym_mode && !strcmp(sym_mode, "plan")) ? kPlan : kTiles;
+  if (diagonals)
+    M->mode = M->sym ? kDiaSym : kDia;
+  else if (!M->sym || sym_full)
+    M->mode = kGather;
+  else
+    M->mode = sym_mode && !strcmp(sym_mode, "plan") ? kPlan : kTiles;
   auto choose_grid = [&]() -> int {
     if (int rc = mode_occupancy(M->mode, per_sm)) return rc;
     if (per_sm < 1) return fail(GBCG_ERR_CUDA, "the persistent solver kernel cannot be resident");
@@ -1043,7 +1053,8 @@ int gbcg_create(gbcg_matrix_t* out, int32_t format, int64_t n, int64_t nnz, cons
   const size_t nn = (size_t)std::max<int64_t>(n, 1);
   TRY(dalloc(&M->r, nn, B));
   // the diagonal layout's product reads p beyond its ends (padding values there): zeros that stay zeros
-  const size_t halo = !diagonals ? 0 : (std::max<int64_t>(-M->dia<double>().lo, M->dia<double>().hi) + kDiaHalo + 63) & ~int64_t(63);
+  const DiaDev<double> dd = M->dia<double>();
+  const size_t halo = diagonals ? (std::max<int64_t>(-dd.lo, dd.hi) + kDiaHalo + 63) & ~int64_t(63) : 0;
   TRY(dalloc(&M->p_base, nn + 2 * halo, B));
   TRY(dalloc(&M->p32_base, nn + 2 * halo, B));
   if (cudaMemsetAsync(M->p_base, 0, sizeof(double) * (nn + 2 * halo), s) != cudaSuccess ||
